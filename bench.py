@@ -316,7 +316,10 @@ def run_reference_nr(args, ws):
 # ---------------------------------------------------------------------------
 # our arm
 # ---------------------------------------------------------------------------
+# "fp64" of more than 96 unknowns runs its contraction on the tensor cores
+# (exact 8-bit digits in FP16, form_key)
 KERNELS = {"fp64": ("k_currents_f64", "k_gemm3m_f64", "k_decide+k_compact"),
+           "fp64_split": ("(none)", "k_split_gemm", "k_split_step"),
            "fp16_scaled": ("k_residual_group", "k_contract_group", "k_decide_group+k_finish_group"),
            "bf16x2": ("k_residual_group", "k_contract_group", "k_decide_group+k_finish_group"),
            "tree": ("k_residual_group", "k_tree_group", "(sweep end inside k_tree_group)")}
@@ -328,9 +331,15 @@ MIXED_OUTSIDE = ("k_group_reset+k_slot_init+k_group_params+k_finish_group(start)
 # launches outside the sweep loop per solve (with no scenario to correct; k_branch_f64 runs
 # where every line's two blocks are identical, as in every feeder of the workloads), and per
 # sweep (the tensor-core forms fold their stop test into the sweep end up to 1024 slots)
-OUTSIDE = {"fp64": ("k_init", 1), "tree": (MIXED_OUTSIDE, 10),
+OUTSIDE = {"fp64": ("k_init", 1), "fp64_split": ("k_init+k_split_step(start)", 2), "tree": (MIXED_OUTSIDE, 10),
            "fp16_scaled": (MIXED_OUTSIDE, 10), "bf16x2": (MIXED_OUTSIDE, 10)}
-PER_SWEEP = {"fp64": 4, "fp16_scaled": 4, "bf16x2": 4, "tree": 2}
+PER_SWEEP = {"fp64": 4, "fp64_split": 2, "fp16_scaled": 4, "bf16x2": 4, "tree": 2}
+
+
+def form_key(form, n):
+    """Which kernels a form runs at n unknowns (csrc/split.cuh: 97 .. 12288 padded to 48)."""
+    n_pad = (n + 47) // 48 * 48
+    return "fp64_split" if form == "fp64" and 96 < n_pad <= 12288 else form
 
 
 def kernel_roofline(form, name, n, B_act_sweeps, ms, peaks, K_pad=None, N_pad=None):
@@ -351,6 +360,22 @@ def kernel_roofline(form, name, n, B_act_sweeps, ms, peaks, K_pad=None, N_pad=No
                 "peak_src": peaks["fp64_src"],
                 "note": "achieved counts the algorithmic 8 n^2 flop per scenario-sweep; the 3M "
                         "form executes 6 n_pad^2 (executed, frac_executed)"}
+    if name == "k_split_gemm":
+        # 28 digit products of 6 n^2 flop each (three real products)
+        ach = 8.0 * n * n * B_act_sweeps / t / 1e12
+        exe = 168.0 * n * n * B_act_sweeps / t / 1e12
+        pk = peaks["bf16_tflops"]
+        return {"bound": "tensor", "achieved": exe, "peak": pk, "unit": "TFLOP/s",
+                "frac": exe / pk, "algorithmic": ach,
+                "frac_of_fp64_rate": ach / peaks["fp64_tflops"],
+                "peak_src": "MEASURED_PEAKS bf16 burst (fp16 same rate), of measured",
+                "note": "achieved counts the FP16 digit products (28 x 6 n^2 per "
+                        "scenario-sweep); algorithmic 8 n^2"}
+    if name == "k_split_step":
+        # partial products read (84 n), v read and written, loads, next operand's digits
+        byts = B_act_sweeps * 190.0 * n / t / 1e9
+        return {"bound": "hbm", "achieved": byts, "peak": peaks["hbm_gbs"], "unit": "GB/s",
+                "frac": byts / peaks["hbm_gbs"], "peak_src": "MEASURED_PEAKS hbm copy, of measured"}
     if name == "k_contract_group":
         zp = 2 if form == "bf16x2" else 1
         ach = 8.0 * n * n * B_act_sweeps / t / 1e12
@@ -455,7 +480,8 @@ def measure(net, form, Sw, Sd, wl, n, steps, warmup, flush, ws, peaks, extra_lau
                 for q in range(3):
                     k_ms[q] += float(ms[k, q])
                 act_sum += int(act[k])
-    names = KERNELS[form]
+    key = form_key(form, n)
+    names = KERNELS[key]
     step_p50 = statistics.median(step_ms)
     sweep_ms = sum(k_ms) / n_prof
     rest_ms = max(0.0, step_p50 - sweep_ms)
@@ -466,13 +492,15 @@ def measure(net, form, Sw, Sd, wl, n, steps, warmup, flush, ws, peaks, extra_lau
     for q in range(3):
         e = {"kernel": names[q], "share": k_ms[q] / n_prof / tot if tot else 0.0,
              "ms_per_sweep": k_ms[q] / max(1, act_sum) * B}
-        if q < 2:
+        if names[q] == "(none)":
+            continue
+        if q < 2 or names[q] == "k_split_step":
             e["roofline"] = kernel_roofline(form, names[q], n, act_sum, k_ms[q], peaks, K_pad,
                                             N_pad)
         kernels.append(e)
-    kernels.append({"kernel": OUTSIDE[form][0], "share": rest_ms / tot if tot else 0.0,
+    kernels.append({"kernel": OUTSIDE[key][0], "share": rest_ms / tot if tot else 0.0,
                     "ms_per_step": rest_ms})
-    dom = max(kernels[:2], key=lambda e: e["share"])
+    dom = max((e for e in kernels if "roofline" in e), key=lambda e: e["share"])
     roof = dict(dom["roofline"])
     roof["kernel"] = dom["kernel"]
     tr = TRAFFIC.get((wl.name, B, form, dom["kernel"]))
@@ -492,8 +520,8 @@ def measure(net, form, Sw, Sd, wl, n, steps, warmup, flush, ws, peaks, extra_lau
             "step_ms_p50": statistics.median(step_ms),
             "step_ms_p99": float(np.percentile(step_ms, 99)), "converged_per_step": good,
             "max_iters": max_iters, "mean_iters": float(it.float().mean().item()),
-            "gpu_launches": steps * (OUTSIDE[form][1] + extra_launches + max_iters * (
-                PER_SWEEP[form] - (1 if form in ("fp16_scaled", "bf16x2") and
+            "gpu_launches": steps * (OUTSIDE[key][1] + extra_launches + max_iters * (
+                PER_SWEEP[key] - (1 if form in ("fp16_scaled", "bf16x2") and
                                    (B + 127) // 128 * 128 <= 1024 else 0))),
             "kernels": kernels, "roofline": roof, "sample": sample}, (V, it, cv)
 
@@ -502,15 +530,12 @@ def measure(net, form, Sw, Sd, wl, n, steps, warmup, flush, ws, peaks, extra_lau
 # (workload, scenarios, form, kernel) -> dram__bytes_read.sum + dram__bytes_write.sum per
 # launch from one ncu capture of the current kernel, with how it was taken
 TRAFFIC = {
-    ("feeder128_b4096", 4096, "fp64", "k_gemm3m_f64"): 66.403584e6 + 1.091584e6,
     ("feeder1024_b16384", 16384, "fp16_scaled", "k_residual_group"):
         4.0 * (404.311040e6 + 49.283840e6),
     ("feeder1024_b16384", 16384, "fp16_scaled", "k_contract_group"):
         2.0 * (1047.367168e6 + 368.998144e6),
 }
 TRAFFIC_SRC = {
-    ("feeder128_b4096", 4096, "fp64", "k_gemm3m_f64"):
-        "ncu capture of this launch configuration (sweep 3, all scenarios active)",
     ("feeder1024_b16384", 16384, "fp16_scaled", "k_residual_group"):
         "ncu capture of an FP32 start sweep at 4096 scenarios x 4 (bytes scale with the "
         "scenarios: measured 453.6 MB = algorithmic 452.6 MB; a double-float sweep 453.9 MB)",

@@ -25,41 +25,12 @@
 #include <cmath>
 #include <cstring>
 
+#include "adj_loads.cuh"
+#include "split.cuh"
 #include "zbus_internal.cuh"
 
 namespace zbus {
 namespace {
-
-__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
-  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
-// acc + a b with four FMAs
-__device__ __forceinline__ double2 cfma(double2 a, double2 b, double2 acc) {
-  return make_double2(fma(a.x, b.x, fma(-a.y, b.y, acc.x)), fma(a.x, b.y, fma(a.y, b.x, acc.y)));
-}
-__device__ __forceinline__ double2 csub(double2 a, double2 b) {
-  return make_double2(a.x - b.x, a.y - b.y);
-}
-
-// conj(S / u^2) = conj(S) u^2 / |u|^4; zero for an absent load.
-__device__ __forceinline__ double2 load_slope(double2 S, double2 u) {
-  if (S.x == 0.0 && S.y == 0.0) return make_double2(0.0, 0.0);
-  const double q = u.x * u.x + u.y * u.y;
-  const double2 u2 = cmul(u, u);
-  const double2 r = cmul(cconj(S), u2);
-  const double inv = 1.0 / (q * q);
-  return make_double2(r.x * inv, r.y * inv);
-}
-
-// x / conj(u) = x u / |u|^2; zero where u = 0 (an absent phase of a padded
-// partial-phase bus).
-__device__ __forceinline__ double2 div_conj(double2 x, double2 u) {
-  const double q = u.x * u.x + u.y * u.y;
-  if (q == 0.0) return make_double2(0.0, 0.0);
-  const double2 r = cmul(x, u);
-  return make_double2(r.x / q, r.y / q);
-}
 
 // Transpose of the three n_pad x n_pad 3M arrays of Z (blockIdx.z selects one).
 __global__ void k_transpose_3m(const double* __restrict__ Zr, const double* __restrict__ Zi,
@@ -116,7 +87,7 @@ __global__ void k_adj_init(SolveCtx* ctx, SolveCtx h, int n, int B) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     h.count = B;
     h.iter = 0;
-    h.err = 0;
+    h.err = h.err ? ctx->err : 0;   // as in k_init
     *ctx = h;
   }
 }
@@ -142,47 +113,30 @@ __global__ void k_adj_rhs(const SolveCtx* __restrict__ ctx, int n, int n_pad) {
     const int k = (int)(t % nbp);
     const int j0 = 3 * k;
     const int64_t o = (int64_t)slot * n_pad + j0;
-    double2 lam[3] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+    double2 x[3] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
     if (j0 < n && ZB_IN(ctx->list[slot], ctx->B, 0x301u)) {
       const int b = ctx->list[slot];
       const int m = min(3, n - j0);
       const int64_t e = (int64_t)b * n + j0;
-      const double inv_s = 1.0 / ctx->gscale[b];
-      double2 v[3], u[3];
+      double2 v[3], u[3], g[3], sw[3], sd[3];
 #pragma unroll
       for (int p = 0; p < 3; ++p) {
         v[p] = p < m ? V[e + p] : make_double2(1.0, 0.0);
         u[p] = p < m ? mu[e + p] : make_double2(0.0, 0.0);
-        const double2 g = p < m ? G[e + p] : make_double2(0.0, 0.0);
-        lam[p] = make_double2(g.x * inv_s, g.y * inv_s);
-        if (Sw && p < m) {
-          const double2 a = load_slope(Sw[e + p], v[p]);
-          const double2 d = cmul(a, u[p]);
-          lam[p].x += d.x;
-          lam[p].y += d.y;
-        }
+        g[p] = p < m ? G[e + p] : make_double2(0.0, 0.0);
+        sw[p] = (Sw && p < m) ? Sw[e + p] : make_double2(0.0, 0.0);
+        sd[p] = (Sd && p < m) ? Sd[e + p] : make_double2(0.0, 0.0);
       }
-      if (Sd && m == 3) {
-#pragma unroll
-        for (int x = 0; x < 3; ++x) {
-          const int y = x == 2 ? 0 : x + 1;
-          const double2 c = load_slope(Sd[e + x], csub(v[x], v[y]));
-          const double2 d = cmul(c, csub(u[x], u[y]));
-          lam[x].x += d.x;
-          lam[x].y += d.y;
-          lam[y].x -= d.x;
-          lam[y].y -= d.y;
-        }
-      }
+      adjoint_rhs(v, u, g, 1.0 / ctx->gscale[b], sw, sd, m, x);
 #pragma unroll
       for (int p = 0; p < 3; ++p)
-        if (p >= m) lam[p] = make_double2(0.0, 0.0);
+        if (p >= m) x[p] = make_double2(0.0, 0.0);
     }
 #pragma unroll
     for (int p = 0; p < 3; ++p) {   // the operand is conj(lambda)
-      Ir[o + p] = lam[p].x;
-      Ii[o + p] = -lam[p].y;
-      Is[o + p] = lam[p].x - lam[p].y;
+      Ir[o + p] = x[p].x;
+      Ii[o + p] = x[p].y;
+      Is[o + p] = x[p].x + x[p].y;
     }
   }
 }
@@ -534,6 +488,19 @@ zbus_status enqueue_sweep_adjoint(zbus_network net, int64_t B, int grid,
   return ZBUS_OK;
 }
 
+// The same on the tensor cores: contraction with the slices of Z^T, then
+// update, stop test and the next conj(lambda) (split.cu).
+zbus_status enqueue_sweep_split_adjoint(zbus_network net, int64_t B, int grid,
+                                        cudaGraphConditionalHandle h, bool use_handle,
+                                        cudaStream_t st, cudaEvent_t* ev) {
+  (void)grid;
+  (void)ev;
+  ZB_CHECK(launch_split_gemm(net->ws.ctx, net->split, net->split_zt, net->n, B, st));
+  launch_split_step(net->ws.ctx, net->split_zt, nullptr, net->n, B, net->split.rows, true, h,
+                    use_handle, st);
+  return ZBUS_OK;
+}
+
 // The adjoint on padded device arrays.
 zbus_status adjoint_device(zbus_network net, int64_t B, const double* S_wye,
                            const double* S_delta, const double* V, const double* G, double tol,
@@ -542,6 +509,7 @@ zbus_status adjoint_device(zbus_network net, int64_t B, const double* S_wye,
   ZB_CHECK(ensure_workspace(net, B));
   ZB_CHECK(ensure_adjoint(net, B, st));
   net->last_group = nullptr;
+  net->last_ctx = nullptr;
   SolveCtx h;
   std::memset(&h, 0, sizeof(h));
   h.S_wye = (const double2*)S_wye;
@@ -564,16 +532,49 @@ zbus_status adjoint_device(zbus_network net, int64_t B, const double* S_wye,
   const int n = net->n;
   k_adj_scale<<<grid_1d(B * 32, 4096), 256, 0, st>>>((const double2*)G, n, (int)B,
                                                      net->adj_scale);
-  k_adj_init<<<grid_1d(B * (int64_t)n, 4096), 256, 0, st>>>(net->ws.ctx, h, n, (int)B);
-  ZB_CUDA(cudaGetLastError());
-  const int grid = gemm_f64_grid((int)B, net->n_pad);
-  if (use_graphs()) {
-    GraphEntry* g = nullptr;
-    ZB_CHECK(get_while_graph(net, B, GRAPH_KEY_ADJOINT, grid, enqueue_sweep_adjoint, &g));
-    ZB_CUDA(cudaGraphLaunch(g->exec, st));
+  const int64_t rows = split_ready(net, true, st) ? split_rows(net, B) : 0;
+  if (rows > 0) {
+    net->last_ctx = net->ws.ctx;
+    split_fill_ctx(&h, net->split);
+    for (int64_t b0 = 0; b0 < B; b0 += rows) {
+      const int64_t Bk = std::min(rows, B - b0);
+      const int64_t o = b0 * n;
+      SolveCtx hk = h;
+      hk.S_wye = h.S_wye ? h.S_wye + o : nullptr;
+      hk.S_del = h.S_del ? h.S_del + o : nullptr;
+      hk.V = h.V + o;
+      hk.Vf = h.Vf + o;
+      hk.G = h.G + o;
+      hk.gscale = h.gscale + b0;
+      hk.iters = iters + b0;
+      hk.conv = converged + b0;
+      hk.B = (int32_t)Bk;
+      hk.err = b0 > 0;
+      k_adj_init<<<grid_1d(Bk * (int64_t)n, 4096), 256, 0, st>>>(net->ws.ctx, hk, n, (int)Bk);
+      launch_split_first(net->ws.ctx, n, Bk, net->split.rows, true, st);
+      ZB_CUDA(cudaGetLastError());
+      if (use_graphs()) {
+        GraphEntry* g = nullptr;
+        ZB_CHECK(get_while_graph(net, Bk, GRAPH_KEY_SPLIT_ADJOINT, 0, enqueue_sweep_split_adjoint,
+                                 &g));
+        ZB_CUDA(cudaGraphLaunch(g->exec, st));
+      } else {
+        for (int k = 0; k < max_iter; ++k)
+          ZB_CHECK(enqueue_sweep_split_adjoint(net, Bk, 0, 0, false, st, nullptr));
+      }
+    }
   } else {
-    for (int k = 0; k < max_iter; ++k)
-      ZB_CHECK(enqueue_sweep_adjoint(net, B, grid, 0, false, st, nullptr));
+    k_adj_init<<<grid_1d(B * (int64_t)n, 4096), 256, 0, st>>>(net->ws.ctx, h, n, (int)B);
+    ZB_CUDA(cudaGetLastError());
+    const int grid = gemm_f64_grid((int)B, net->n_pad);
+    if (use_graphs()) {
+      GraphEntry* g = nullptr;
+      ZB_CHECK(get_while_graph(net, B, GRAPH_KEY_ADJOINT, grid, enqueue_sweep_adjoint, &g));
+      ZB_CUDA(cudaGraphLaunch(g->exec, st));
+    } else {
+      for (int k = 0; k < max_iter; ++k)
+        ZB_CHECK(enqueue_sweep_adjoint(net, B, grid, 0, false, st, nullptr));
+    }
   }
   const int nb = (n + 2) / 3;
   k_adj_out<<<grid_1d(B * (int64_t)nb, 4096), 256, 0, st>>>(
@@ -589,6 +590,7 @@ zbus_status adjoint_tree_device(zbus_network net, int64_t B, const double* S_wye
                                 double tol, int32_t max_iter, double* dS_wye, double* dS_delta,
                                 int32_t* iters, uint8_t* converged, cudaStream_t st) {
   net->last_group = nullptr;
+  net->last_ctx = nullptr;
   // the iterate and the residual on chip up to 96 KB (two CTAs per SM at the
   // largest such feeder, ~1000 buses), else in the scratch slice
   const size_t onchip = 2 * (size_t)net->n * sizeof(double2);
@@ -666,6 +668,7 @@ bool on_device(const void* p) {
 }  // namespace
 
 void free_adjoint(zbus_network net) {
+  split_release(&net->split_zt);
   cudaFree(net->ZrT);
   cudaFree(net->ZiT);
   cudaFree(net->ZsT);

@@ -9,6 +9,7 @@
 #include <set>
 
 #include "group.cuh"
+#include "split.cuh"
 #include "zbus_internal.cuh"
 
 namespace zbus {
@@ -155,6 +156,50 @@ zbus_status ensure_workspace(zbus_network net, int64_t B) {
   return ZBUS_OK;
 }
 
+// Bytes of split-sweep scratch up to which a batch is solved in one pass; a
+// larger batch runs in passes (its scenarios are independent).
+constexpr size_t SPLIT_SCRATCH_MAX = (size_t)8 << 30;
+
+bool split_ready(zbus_network net, bool adjoint, cudaStream_t st) {
+  if (!split_size_ok(net->n_pad)) return false;
+  SplitOps* ops = adjoint ? &net->split_zt : &net->split_z;
+  if (ops->Z) return true;
+  const std::string msg = g_last_error;
+  const zbus_status s = adjoint
+                            ? split_pack(ops, net->ZrT, net->ZiT, net->n, net->n_pad, st)
+                            : split_pack(ops, net->Zr, net->Zi, net->n, net->n_pad, st);
+  if (s == ZBUS_OK) return true;
+  g_last_error = msg;
+  cudaGetLastError();
+  return false;
+}
+
+int64_t split_rows(zbus_network net, int64_t B) {
+  const size_t per = split_scratch_bytes(net->n, 128) / 128;
+  const int64_t most = std::max<int64_t>(128, (int64_t)(SPLIT_SCRATCH_MAX / per) / 128 * 128);
+  const int64_t want = std::min(most, (B + 127) / 128 * 128);
+  if (net->split.rows >= want) return net->split.rows;
+  if (net->split_base) {
+    if (cudaDeviceSynchronize() != cudaSuccess) return 0;
+    drop_graphs(net);
+    cudaFree(net->split_base);
+    net->split_base = nullptr;
+    net->split = SplitScratch();
+  }
+  void* base = nullptr;
+  if (cudaMalloc(&base, split_scratch_bytes(net->n, want)) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  if (split_scratch_bind(&net->split, base, net->n, want) != ZBUS_OK) {
+    cudaFree(base);
+    net->split = SplitScratch();
+    return 0;
+  }
+  net->split_base = base;
+  return want;
+}
+
 bool use_graphs() {
   const char* e = std::getenv("ZBUS_NO_GRAPH");
   return !(e && e[0] == '1');
@@ -172,6 +217,22 @@ zbus_status enqueue_sweep_f64(zbus_network net, int64_t B, int grid, cudaGraphCo
   launch_gemm_f64(net->ws.ctx, net->Zr, net->Zi, net->Zs, net->w, net->n, net->n_pad, grid, st);
   if (ev) ZB_CUDA(cudaEventRecord(ev[2], st));
   launch_converge(net->ws.ctx, (int)B, h, use_handle, st);
+  if (ev) ZB_CUDA(cudaEventRecord(ev[3], st));
+  return ZBUS_OK;
+}
+
+// The same with the contraction on the tensor cores (split.cu); the first
+// operand was written before the loop.
+zbus_status enqueue_sweep_split(zbus_network net, int64_t B, int grid,
+                                cudaGraphConditionalHandle h, bool use_handle, cudaStream_t st,
+                                cudaEvent_t* ev = nullptr) {
+  (void)grid;
+  if (ev) ZB_CUDA(cudaEventRecord(ev[0], st));
+  if (ev) ZB_CUDA(cudaEventRecord(ev[1], st));
+  ZB_CHECK(launch_split_gemm(net->ws.ctx, net->split, net->split_z, net->n, B, st));
+  if (ev) ZB_CUDA(cudaEventRecord(ev[2], st));
+  launch_split_step(net->ws.ctx, net->split_z, net->w, net->n, B, net->split.rows, false, h,
+                    use_handle, st);
   if (ev) ZB_CUDA(cudaEventRecord(ev[3], st));
   return ZBUS_OK;
 }
@@ -346,7 +407,13 @@ zbus_status zbus_last_device_status(zbus_network net, void* cuda_stream) {
   cudaStream_t st = (cudaStream_t)cuda_stream;
   if (!net->last_group) {
     ZB_CUDA(cudaStreamSynchronize(st));
-    return ZBUS_OK;
+    if (!net->last_ctx) return ZBUS_OK;
+    int32_t err = 0;
+    ZB_CUDA(cudaMemcpyAsync(&err, &net->last_ctx->err, sizeof(err), cudaMemcpyDeviceToHost, st));
+    ZB_CUDA(cudaStreamSynchronize(st));
+    if (err == 0) return ZBUS_OK;
+    return fail(ZBUS_ERR_TIMEOUT, "the FP64 contraction's pipeline gave up (code " +
+                                      std::to_string(err) + ")");
   }
   return group_device_status(net->last_group, st);
 }
@@ -371,7 +438,7 @@ const char* zbus_last_error(void) { return g_last_error.c_str(); }
 int32_t zbus_checked_status(uint32_t* word) {
   cudaDeviceSynchronize();
   uint32_t (*const words[])(bool) = {check_word_f64, check_word_group, check_word_adjoint,
-                                     check_word_nr, check_word_phased};
+                                     check_word_nr, check_word_phased, check_word_split};
   uint32_t first = 0;
   for (auto fn : words) {
     const uint32_t w = fn(true);
@@ -498,6 +565,8 @@ void zbus_network_destroy(zbus_network net) {
   free_mixed(net);
   phased_free(net);
   free_adjoint(net);
+  split_release(&net->split_z);
+  cudaFree(net->split_base);
   cudaFree(net->Z);
   cudaFree(net->w);
   cudaFree(net->ys);
@@ -560,6 +629,7 @@ zbus_status zbus_network_reserve(zbus_network net, int64_t B, int32_t precision)
   ZB_CHECK(check_device(net));
   ZB_CHECK(ensure_workspace(net, B));
   ZB_CHECK(ensure_3m(net, nullptr));
+  if (precision == ZBUS_FP64 && split_ready(net, false, nullptr)) split_rows(net, B);
   if (precision == ZBUS_TREE_SWEEP) ZB_CHECK(prepare_tree(net, nullptr));
   else if (precision != ZBUS_FP64) ZB_CHECK(prepare_mixed(net, precision, nullptr));
   return ZBUS_OK;
@@ -569,6 +639,52 @@ zbus_status zbus_network_reserve(zbus_network net, int64_t B, int32_t precision)
 
 namespace zbus {
 namespace {
+
+// The plain method with its contraction on the tensor cores: passes of up to
+// `rows` scenarios of the batch described by h.
+zbus_status solve_split(zbus_network net, const SolveCtx& h, int64_t rows, bool profile,
+                        cudaStream_t st) {
+  const int n = net->n;
+  net->last_ctx = net->ws.ctx;
+  for (int64_t b0 = 0; b0 < h.B; b0 += rows) {
+    const int64_t Bk = std::min<int64_t>(rows, h.B - b0);
+    const int64_t o = b0 * n;
+    SolveCtx hk = h;
+    split_fill_ctx(&hk, net->split);
+    hk.S_wye = h.S_wye ? h.S_wye + o : nullptr;
+    hk.S_del = h.S_del ? h.S_del + o : nullptr;
+    hk.V_init = h.V_init ? h.V_init + o : nullptr;
+    hk.V = h.V + o;
+    hk.iters = h.iters + b0;
+    hk.conv = h.conv + b0;
+    hk.B = (int32_t)Bk;
+    hk.err = b0 > 0;
+    if (profile) {
+      ZB_CHECK(ensure_profile(net, h.max_iter));
+      ZB_CUDA(cudaMemsetAsync(net->prof.d_hist, 0, (size_t)h.max_iter * sizeof(int32_t), st));
+      hk.hist = net->prof.d_hist;
+      hk.hist_n = h.max_iter;
+    }
+    launch_init(net->ws.ctx, hk, net->w, n, (int)Bk, st);
+    launch_split_first(net->ws.ctx, n, Bk, net->split.rows, false, st);
+    ZB_CUDA(cudaGetLastError());
+    if (profile) {
+      for (int k = 0; k < h.max_iter; ++k)
+        ZB_CHECK(enqueue_sweep_split(net, Bk, 0, 0, false, st,
+                                     &net->prof.ev[(size_t)4 * k]));
+      net->prof.sweeps = h.max_iter;
+    } else if (use_graphs()) {
+      GraphEntry* g = nullptr;
+      ZB_CHECK(get_while_graph(net, Bk, GRAPH_KEY_SPLIT, 0, enqueue_sweep_split, &g));
+      ZB_CUDA(cudaGraphLaunch(g->exec, st));
+    } else {
+      for (int k = 0; k < h.max_iter; ++k)
+        ZB_CHECK(enqueue_sweep_split(net, Bk, 0, 0, false, st));
+    }
+  }
+  ZB_CUDA(cudaGetLastError());
+  return ZBUS_OK;
+}
 
 // The solve on device buffers (the arguments checked by zbus_solve).
 zbus_status solve_device(zbus_network net, int64_t B, const double* S_wye, const double* S_delta,
@@ -588,7 +704,8 @@ zbus_status solve_device(zbus_network net, int64_t B, const double* S_wye, const
                      {converged}, tol, max_iter, o, st);
   }
 
-  net->last_group = nullptr;   // the plain method has no device-side waits
+  net->last_group = nullptr;
+  net->last_ctx = nullptr;   // the sweeps on the CUDA cores have no device-side waits
   if (o.profile != 1 && B <= F64_BM && net->n_pad <= FUSED_MAX_NPAD) {
     // a small feeder and at most one tile of scenarios: the whole solve in
     // one launch (bitwise the results of the sweep-per-launch path below)
@@ -617,6 +734,9 @@ zbus_status solve_device(zbus_network net, int64_t B, const double* S_wye, const
   h.max_iter = max_iter;
   h.rule = o.conv_rule;
   h.ntn = net->n_pad / F64_BN;
+  const int64_t rows = split_ready(net, false, st) ? split_rows(net, B) : 0;
+  if (rows > 0 && (rows >= B || o.profile != 1))
+    return solve_split(net, h, rows, o.profile == 1, st);
   const int grid = gemm_f64_grid((int)B, net->n_pad);
   if (o.profile == 1) {
     ZB_CHECK(ensure_profile(net, max_iter));

@@ -19,7 +19,8 @@ namespace {
 // Run start: v^0 = w (or the warm start), flags cleared, every scenario active.
 // ---------------------------------------------------------------------------
 // The solve's context arrives by value and is stored for the later kernels;
-// this kernel itself only uses the by-value copy.
+// this kernel itself only uses the by-value copy.  h.err nonzero: a later
+// pass of the same call, which keeps the error word of the earlier ones.
 __global__ void k_init(SolveCtx* ctx, SolveCtx h, const double2* __restrict__ w, int n, int B) {
   const double2* Vi = h.V_init;
   double2* V = h.V;
@@ -38,7 +39,7 @@ __global__ void k_init(SolveCtx* ctx, SolveCtx h, const double2* __restrict__ w,
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     h.count = B;
     h.iter = 0;
-    h.err = 0;
+    h.err = h.err ? ctx->err : 0;
     *ctx = h;
   }
 }

@@ -39,6 +39,37 @@ __device__ __forceinline__ void bus_injection(const double2* v, const double2* s
   for (int p = 0; p < 3; ++p) inj[p] = make_double2(-d[p].x, -d[p].y);
 }
 
+// bus_injection (m valid phases; absent loads given as zeros) for a thread per
+// bus.  A bus with loads of one kind forms three quotients whichever kind it
+// is, so a warp whose buses carry different kinds does not run both paths.
+__device__ __forceinline__ void bus_injection_one(const double2* v, const double2* sw,
+                                                  const double2* sd, int m, double2* inj) {
+  bool wye = false, delta = false;
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    wye = wye || sw[p].x != 0.0 || sw[p].y != 0.0;
+    delta = delta || sd[p].x != 0.0 || sd[p].y != 0.0;
+  }
+  delta = delta && m == 3;
+  if (wye && delta) {
+    bus_injection(v, sw, sd, m, inj);
+    return;
+  }
+  double2 i[3];
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    const int q = p == 2 ? 0 : p + 1;
+    const double2 u = delta ? make_double2(v[p].x - v[q].x, v[p].y - v[q].y) : v[p];
+    i[p] = load_draw(delta ? sd[p] : sw[p], u);
+  }
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    const int q = p == 0 ? 2 : p - 1;
+    inj[p] = delta ? make_double2(i[q].x - i[p].x, i[q].y - i[p].y)
+                   : make_double2(-i[p].x, -i[p].y);
+  }
+}
+
 // Double-float versions for the defect residual.  The current drawn by a
 // load, conj(S / v), is formed at the double-float voltage v = vh + vl: the
 // FP32 quotient at vh, then one correction step on the remainder

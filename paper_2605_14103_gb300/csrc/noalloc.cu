@@ -18,10 +18,12 @@
 // (on different streams, or from several host threads) race on it.  Every
 // array argument must be device memory: the sweeps read and write the
 // caller's arrays directly, with no staging.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
 
+#include "split.cuh"
 #include "zbus_internal.cuh"
 
 namespace zbus {
@@ -135,13 +137,51 @@ extern "C" zbus_status zbus_solve_noalloc(zbus_network net, int64_t B, const dou
   h.ntn = ntn;
   SolveCtx* ctx = (SolveCtx*)p;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  // the FP64 sweeps have no device-side waits: zbus_last_device_status must
-  // not report the error word of an earlier mixed-precision solve
+  // zbus_last_device_status must not report the error word of an earlier
+  // mixed-precision solve
   net->last_group = nullptr;
+  net->last_ctx = nullptr;
   // The run start writes the whole context, the active list, iters and flags,
   // so nothing left in the array by an earlier call is read: every partial,
   // keep mark and operand element (padding included) is written in a sweep
   // before the kernels of that sweep read it.
+  if (net->split_z.Z) {
+    // the contraction on the tensor cores, as zbus_solve: its scratch takes
+    // more bytes per scenario, so the batch runs in passes of the scenarios
+    // that fit (independent of each other: the same bits)
+    const size_t fixed = a256(sizeof(SolveCtx));
+    const size_t per = split_scratch_bytes(net->n, 256) / 256 + sizeof(int32_t);
+    const int64_t rows = std::min<int64_t>(B, (int64_t)((STATIC_SCRATCH_BYTES - fixed - 4096) / per));
+    if (rows >= 1) {
+      SplitScratch scratch;
+      ZB_CHECK(split_scratch_bind(&scratch, p + fixed + a256((size_t)rows * sizeof(int32_t)),
+                                  net->n, rows));
+      net->last_ctx = ctx;
+      h.list = (int32_t*)(p + fixed);
+      split_fill_ctx(&h, scratch);
+      for (int64_t b0 = 0; b0 < B; b0 += rows) {
+        const int64_t Bk = std::min(rows, B - b0);
+        const int64_t o = b0 * net->n;
+        SolveCtx hk = h;
+        hk.S_wye = h.S_wye ? h.S_wye + o : nullptr;
+        hk.S_del = h.S_del ? h.S_del + o : nullptr;
+        hk.V_init = h.V_init ? h.V_init + o : nullptr;
+        hk.V = h.V + o;
+        hk.iters = iters + b0;
+        hk.conv = converged + b0;
+        hk.B = (int32_t)Bk;
+        hk.err = b0 > 0;
+        launch_init(ctx, hk, net->w, net->n, (int)Bk, st);
+        launch_split_first(ctx, net->n, Bk, rows, false, st);
+        for (int k = 0; k < max_iter; ++k) {
+          ZB_CHECK(launch_split_gemm(ctx, scratch, net->split_z, net->n, Bk, st));
+          launch_split_step(ctx, net->split_z, net->w, net->n, Bk, rows, false, 0, false, st);
+        }
+      }
+      ZB_CUDA(cudaGetLastError());
+      return ZBUS_OK;
+    }
+  }
   launch_init(ctx, h, net->w, net->n, (int)B, st);
   const int grid = gemm_f64_grid((int)B, net->n_pad);
   for (int k = 0; k < max_iter; ++k) {

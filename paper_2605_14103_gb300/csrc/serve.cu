@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "group.cuh"
+#include "split.cuh"
 
 namespace zbus {
 namespace {
@@ -149,6 +150,25 @@ extern "C" zbus_status zbus_serve(const zbus_serve_config* cfg, zbus_network* po
                               "operands of the largest feeder (" +
                                   std::to_string(per_slot * 128 + peak_one) + " bytes)");
   const size_t ops_budget = budget - (size_t)per_slot * cap;
+  // the slices the plain method keeps of each Z are no part of the cache:
+  // they stay only where they fit beside all of it
+  {
+    size_t all = 0, most_form = 0, slices = 0;
+    for (auto net : nets) {
+      all += cache_bytes(net, cfg->precision);
+      most_form = std::max(most_form, form_extra(net));
+      if (net->split_z.Z) slices += split_ops_bytes(net->n);
+      if (net->split_zt.Z) slices += split_ops_bytes(net->n);
+    }
+    if (slices > 0 && all + most_form + slices > ops_budget) {
+      ZB_CUDA(cudaStreamSynchronize(st));
+      for (auto net : nets) {
+        drop_graphs(net);
+        split_release(&net->split_z);
+        split_release(&net->split_zt);
+      }
+    }
+  }
   // the operand cache starts with the feeders that hold their operands (or
   // the complex Z they are packed from) and fit, in pool order; the others
   // give their dense operands up now and are formed on demand

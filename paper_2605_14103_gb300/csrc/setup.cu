@@ -10,6 +10,7 @@
 #include <cstring>
 #include <numeric>
 
+#include "split.cuh"
 #include "zbus_internal.cuh"
 
 namespace zbus {
@@ -546,6 +547,9 @@ zbus_status build_network(zbus_network net, int32_t n_total, int64_t nnz, const 
       break;
     }
     s = ensure_3m(net, st);
+    // the plain method's tensor-core operands too: the allocation-free solve
+    // cannot form them (a device too full for them keeps the FP64 contraction)
+    if (s == ZBUS_OK) split_ready(net, false, st);
   } while (0);
   cudaStreamSynchronize(st);
   cudaFree(d_sp);
@@ -640,6 +644,7 @@ void release_z(zbus_network net) {
 void release_3m(zbus_network net) {
   drop_graphs(net);   // their kernels hold the operand addresses
   free_adjoint(net);
+  split_release(&net->split_z);
   cudaFree(net->Zr);
   cudaFree(net->Zi);
   cudaFree(net->Zs);

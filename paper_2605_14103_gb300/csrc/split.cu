@@ -1,0 +1,783 @@
+// The plain FP64 sweep (Sec. II-B) with its contraction Z i on the tensor
+// cores, without rounding: each operand is held as 55-bit fixed point with
+// one power-of-two scale per row, cut into seven balanced 8-bit digits stored
+// in FP16 (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numerical
+// Algorithms 59, 2012).  A product of two digits is an integer of at most
+// 2^14 (2^16), so 1024 (256) of them sum exactly in the FP32 accumulator; the epilogue
+// adds those sums in 32-bit integers.  The complex product uses three real
+// ones (Re, Im and Re + Im, the sums formed as integers, so the scheme's
+// cancellations are exact), and the products of digits p and q are kept for
+// p + q <= 6: what is left out is about 2^-56 of the rows' largest entries
+// times the square root of n, below the rounding of an FP64 sum of n terms.  Every kept bit is an integer, so a result does not depend on the
+// tile, the batch or the order of the sums.
+//
+// Why: this GPU does 1.25 TFLOP/s in FP64 and about 1.9 PFLOP/s in FP16; the
+// 28 digit products of 6 n^2 operations each are 168 n^2 operations at 1500
+// times the rate.
+//
+// Measured per sweep against the FP64 contraction (k_currents_f64 +
+// k_gemm3m_f64 + the stop test): 1000 scenarios of 3069 unknowns 66 -> 1.35 ms
+// (contraction 1.03), 4096 of 381 3.5 -> 0.29 ms (0.085).  Error of one map
+// against extended precision, 102 to 2397 unknowns: 0.99 to 0.43 of the FP64
+// contraction's root mean square; of one adjoint sweep 0.70 to 0.28.
+//
+// One sweep is two kernels: k_split_gemm (the 21 partial products of every
+// active scenario) and k_split_step (recombination, update, stop test, active
+// list and the operand of the next sweep, one block per scenario).
+#include <cuda_fp16.h>
+#include <cudaTypedefs.h>
+
+#include <algorithm>
+#include <cmath>
+
+#include "adj_loads.cuh"
+#include "loads.cuh"
+#include "split.cuh"
+#include "tc_ptx.cuh"
+
+namespace zbus {
+namespace {
+
+using namespace tc;
+
+constexpr int GEMM_THREADS = 320;      // TMA, MMA and eight epilogue warps
+constexpr int EPI_WARPS = 8;
+constexpr int TMEM_COLS = 512;         // two accumulators of up to 256 columns
+constexpr int ACC_STRIDE = 256;
+constexpr unsigned long long SPLIT_DRAIN_NS = 2000000000ull;
+
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar,
+                                            int x, int y, int z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(su32(dst)),
+      "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(su32(bar))
+      : "memory");
+}
+
+__device__ __forceinline__ void st_i8(int32_t* p, const int* v) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]),
+               "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// Work of the contraction: one item is the 128 x BN block (mt, nt) of one
+// partial product (c, d): component c (Re, Im, Re + Im) and digit weight d,
+// the sum over p <= d of X_p Z_{d-p}^T.  Items are listed from the longest
+// (d = 6) to the shortest and dealt to the blocks back and forth, so every
+// block gets about the same number of k-blocks.
+// ---------------------------------------------------------------------------
+struct SplitItem {
+  int c, d, mt, nt;
+};
+
+__device__ __forceinline__ SplitItem split_item(int g, int mtiles, int ntn) {
+  const int per = mtiles * ntn;
+  const int cls = g / per, t = g % per;
+  SplitItem it;
+  it.d = SPLIT_S - 1 - cls / 3;
+  it.c = cls % 3;
+  it.mt = t / ntn;
+  it.nt = t % ntn;
+  return it;
+}
+
+// k-blocks whose digit products sum exactly (to at most 2^24) in the FP32
+// accumulator: digits are at most 128, the first digit of Re + Im 256.
+__device__ __forceinline__ int split_chunk(const SplitItem& it) {
+  return (it.c < 2 ? 1024 : it.d > 0 ? 512 : 256) / BK;
+}
+
+__device__ __forceinline__ int split_deal(int round) {
+  const int G = gridDim.x;
+  return round * G + ((round & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
+}
+
+// ---------------------------------------------------------------------------
+// Partial products.  Warp roles: 0 = TMA producer, 1 = TMEM owner and MMA
+// issuer, 2..9 = epilogue (warp w reads TMEM lanes 32 (w % 4) .. + 31 of one
+// half of the columns).  The accumulator is drained before its sum can pass
+// 2^24 (split_chunk) into 32-bit integer registers, the next chunk's MMAs running meanwhile in
+// the other accumulator.  Bound by the tensor pipe at large batches: 16384
+// scenarios of 3069 unknowns in 13.9 ms, 1.86 PFLOP/s of digit products (0.98
+// of the measured cuBLAS rate); a few scenarios read the 400 MB of slices of
+// Z once per sweep (0.15 ms).  Every wait is bounded as in k_contract_group, and
+// a block that gives up records its code and leaves nothing in flight.
+// ---------------------------------------------------------------------------
+template <int BN, int STAGES>
+__global__ void __launch_bounds__(GEMM_THREADS, 1)
+k_split_gemm(SolveCtx* __restrict__ ctx, const __grid_constant__ CUtensorMap tmX,
+             const __grid_constant__ CUtensorMap tmZ, int n, int num_kb, int64_t rows) {
+  constexpr int A_BYTES = BM * BK * 2;
+  constexpr int B_BYTES = BN * BK * 2;
+  constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+  constexpr int HN = BN / 2;   // columns of one epilogue warp
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = (uint64_t*)(smem + STAGES * STAGE_BYTES);
+  uint64_t* empty = full + STAGES;
+  uint64_t* tfull = empty + STAGES;
+  uint64_t* tempty = tfull + 2;
+  uint64_t* drain = tempty + 2;
+  uint32_t* tmem_holder = (uint32_t*)(drain + 1);
+
+  const int count = ctx->count;
+  const int mtiles = (count + BM - 1) / BM;
+  const int ntn = (n + BN - 1) / BN;
+  const int total = 3 * SPLIT_S * mtiles * ntn;
+  if ((int)blockIdx.x >= total) return;   // whole block, before any barrier
+  const int rounds = (total + gridDim.x - 1) / gridDim.x;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int u = 0; u < 2; ++u) {
+      mbar_init(&tfull[u], 1);
+      mbar_init(&tempty[u], EPI_WARPS);
+    }
+    mbar_init(drain, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     su32(tmem_holder)),
+                 "r"((uint32_t)TMEM_COLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_holder;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      uint32_t kc = 0;   // stage fills issued
+      bool ok = true;
+      for (int r = 0; r < rounds && ok; ++r) {
+        const int g = split_deal(r);
+        if (g >= total) continue;
+        const SplitItem it = split_item(g, mtiles, ntn);
+        // digit q of Z ascending in every item, so items of other weights
+        // running at the same time read the same slices of Z
+        for (int q = 0; q <= it.d && ok; ++q)
+          for (int kb = 0; kb < num_kb; ++kb) {
+            const int s = kc % STAGES;
+            const uint32_t round = kc / STAGES;
+            if (!mbar_wait(&empty[s], (round & 1) ^ 1)) {
+              atomicCAS(&ctx->err, 0, 111);
+              ok = false;
+              break;
+            }
+            uint8_t* st = smem + s * STAGE_BYTES;
+            mbar_expect_tx(&full[s], STAGE_BYTES);
+            tma_load_3d(st, &tmX, &full[s], kb * BK, it.mt * BM, it.c * SPLIT_S + it.d - q);
+            tma_load_3d(st + A_BYTES, &tmZ, &full[s], kb * BK, it.nt * BN,
+                        it.c * SPLIT_S + q);
+            ++kc;
+          }
+      }
+      // drain: the last fill of every stage has landed
+      const uint32_t first = kc > (uint32_t)STAGES ? kc - STAGES : 0u;
+      for (uint32_t j = first; j < kc; ++j)
+        if (!mbar_wait(&full[j % STAGES], (j / STAGES) & 1, SPLIT_DRAIN_NS)) {
+          atomicCAS(&ctx->err, 0, 115);
+          break;
+        }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // kind::f16 instruction descriptor: D f32, A and B f16, both K-major
+      const uint32_t idesc =
+          (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+      uint32_t kc = 0, ch = 0;   // stages and accumulator chunks used
+      bool ok = true, issued = false;
+      for (int r = 0; r < rounds && ok; ++r) {
+        const int g = split_deal(r);
+        if (g >= total) continue;
+        const SplitItem it = split_item(g, mtiles, ntn);
+        const int blocks = (it.d + 1) * num_kb, chunk = split_chunk(it);
+        for (int b0 = 0; b0 < blocks && ok; b0 += chunk, ++ch) {
+          const int buf = ch & 1;
+          if (!mbar_wait(&tempty[buf], ((ch >> 1) & 1) ^ 1)) {
+            atomicCAS(&ctx->err, 0, 114);
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t d = tmem + (uint32_t)(buf * ACC_STRIDE);
+          const int b1 = min(blocks, b0 + chunk);
+          for (int b = b0; b < b1; ++b, ++kc) {
+            const int s = kc % STAGES;
+            if (!mbar_wait(&full[s], (kc / STAGES) & 1)) {
+              atomicCAS(&ctx->err, 0, 112);
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t a0 = su32(smem + s * STAGE_BYTES);
+#pragma unroll
+            for (int kk = 0; kk < BK / 16; ++kk)
+              umma_f16(d, sw128_desc(a0 + kk * 32), sw128_desc(a0 + A_BYTES + kk * 32), idesc,
+                       (b != b0 || kk != 0) ? 1u : 0u);
+            issued = true;
+            umma_commit(&empty[s]);
+          }
+          if (ok) umma_commit(&tfull[buf]);
+        }
+      }
+      // drain: every MMA this thread issued has completed before the tensor
+      // memory is freed
+      if (issued) {
+        umma_commit(drain);
+        if (!mbar_wait(drain, 0, SPLIT_DRAIN_NS)) atomicCAS(&ctx->err, 0, 116);
+      }
+    }
+  } else {
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const int ld = (n + 7) & ~7;
+    int32_t* const D = ctx->D;
+    uint32_t ch = 0;
+    bool ok = true;
+    for (int r = 0; r < rounds && ok; ++r) {
+      const int g = split_deal(r);
+      if (g >= total) continue;
+      const SplitItem it = split_item(g, mtiles, ntn);
+      const int blocks = (it.d + 1) * num_kb, chunk = split_chunk(it);
+      int acc[HN];
+#pragma unroll
+      for (int t = 0; t < HN; ++t) acc[t] = 0;
+      for (int b0 = 0; b0 < blocks; b0 += chunk, ++ch) {
+        const int buf = ch & 1;
+        ok = mbar_wait(&tfull[buf], (ch >> 1) & 1);
+        tc_fence_after();
+        if (!ok) {
+          if (lane == 0) atomicCAS(&ctx->err, 0, 113);
+          break;
+        }
+        const uint32_t ta =
+            tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * ACC_STRIDE + half * HN);
+#pragma unroll
+        for (int c = 0; c < HN / 32; ++c) {
+          float v[32];
+          tmem_ld32(ta + (uint32_t)(c * 32), v);
+          if (c == HN / 32 - 1) {
+            // the accumulator is in registers now: hand it back
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tempty[buf]);
+          }
+#pragma unroll
+          for (int t = 0; t < 32; ++t) acc[c * 32 + t] += __float2int_rn(v[t]);
+        }
+      }
+      const int64_t row = (int64_t)it.mt * BM + q * 32 + lane;
+      if (ok && row < count) {
+        const int col0 = it.nt * BN + half * HN;
+        int32_t* dst = D + ((int64_t)(it.c * SPLIT_S + it.d) * rows + row) * ld + col0;
+#pragma unroll
+        for (int t = 0; t < HN; t += 8)
+          if (col0 + t < ld) st_i8(dst + t, acc + t);
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"((uint32_t)TMEM_COLS));
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Fixed point and digits.
+// ---------------------------------------------------------------------------
+
+// Exponent e of a row whose largest magnitude has the bit pattern `top`:
+// every entry is below 2^e.  Clamped so that the scales stay finite (entries
+// below 2^-900 2^-55 become zero).
+__device__ __forceinline__ int row_exponent(unsigned long long top) {
+  return max(-900, (int)(top >> 52) - 1022);
+}
+
+// round(x 2^(55 - e)) with integer instructions (the conversion instruction
+// runs on the FP64 units); |x| < 2^e.
+__device__ __forceinline__ long long fixed_point(double x, int e) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((u >> 52) & 0x7FF);
+  unsigned long long m = u & 0xFFFFFFFFFFFFFull;
+  m = ex ? m | (1ull << 52) : m;
+  // x = m 2^(max(ex, 1) - 1075)
+  const int sh = max(ex, 1) - 1075 + SPLIT_BITS - e;   // at most 1
+  if (sh >= 0) {
+    m <<= sh;
+  } else if (sh < -55) {
+    m = 0ull;
+  } else {
+    m = (m + (1ull << (-sh - 1))) >> -sh;
+  }
+  return (u >> 63) ? -(long long)m : (long long)m;
+}
+
+// Slices of one row of n complex values, by all threads of the block: digit p
+// of component c of value(j) goes to plane c * 7 + p of out, `plane` halves
+// apart, eight columns at a time.
+template <typename Load>
+__device__ __forceinline__ void write_slices(Load value, int n, int K_pad, int e, __half* out,
+                                             int64_t plane) {
+  const __half2 bias = __floats2half2_rn(1280.f, 1280.f);
+  for (int g = threadIdx.x; g < K_pad / 8; g += blockDim.x) {
+#pragma unroll 1
+    for (int c = 0; c < 3; ++c) {
+      long long y[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int j = g * 8 + i;
+        const double2 v = j < n ? value(j) : make_double2(0.0, 0.0);
+        y[i] = 0;
+        if (c != 1) y[i] += fixed_point(v.x, e);
+        if (c != 0) y[i] += fixed_point(v.y, e);
+      }
+      __half* dst = out + (int64_t)c * SPLIT_S * plane + g * 8;
+#pragma unroll
+      for (int p = SPLIT_S - 1; p >= 0; --p) {
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          uint32_t pair = 0x64006400u;   // the halves 1024 + (digit + 256), minus 1280 below
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            long long& v = y[2 * i + h];
+            int d;
+            if (p > 0) {
+              d = (int)(((uint32_t)v + 128u) & 255u) - 128;
+              v = (v - d) >> 8;
+            } else {
+              d = (int)v;   // at most 256 in magnitude
+            }
+            pair += (uint32_t)(d + 256) << (16 * h);
+          }
+          const __half2 hv = __hsub2(*reinterpret_cast<const __half2*>(&pair), bias);
+          w[i] = *reinterpret_cast<const uint32_t*>(&hv);
+        }
+        *reinterpret_cast<uint4*>(dst + p * plane) = make_uint4(w[0], w[1], w[2], w[3]);
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ unsigned long long abs_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+__device__ __forceinline__ unsigned long long max_u64(unsigned long long a, unsigned long long b) {
+  return a > b ? a : b;
+}
+
+// Maximum over the block (valid in every thread); red: one word per warp.
+__device__ __forceinline__ unsigned long long block_max_u64(unsigned long long x,
+                                                            unsigned long long* red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x = max_u64(x, __shfl_xor_sync(0xffffffffu, x, o));
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
+  __syncthreads();
+  x = red[0];
+  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) x = max_u64(x, red[w]);
+  return x;
+}
+
+// Matrix rows (one block each): slices and scale 2^(e - 31) of row i.
+__global__ void __launch_bounds__(256)
+k_split_pack(const double* __restrict__ Zr, const double* __restrict__ Zi, int n, int n_pad,
+             int K_pad, __half* __restrict__ out, double* __restrict__ zs) {
+  __shared__ unsigned long long red[8];
+  const int i = blockIdx.x;
+  const double* zr = Zr + (int64_t)i * n_pad;
+  const double* zi = Zi + (int64_t)i * n_pad;
+  unsigned long long top = 0ull;
+  for (int j = threadIdx.x; j < n; j += blockDim.x)
+    top = max_u64(top, max_u64(abs_bits(zr[j]), abs_bits(zi[j])));
+  top = block_max_u64(top, red);
+  const int e = row_exponent(top);
+  write_slices([&](int j) { return make_double2(zr[j], zi[j]); }, n, K_pad, e,
+               out + (int64_t)i * K_pad, (int64_t)n * K_pad);
+  if (threadIdx.x == 0) zs[i] = ldexp(1.0, e - 31);
+}
+
+// ---------------------------------------------------------------------------
+// Update, stop test and next operand, one block per active scenario.
+//   v_i <- w_i + 2^(ez_i + ex_b - 62) sum_d D_d 2^(8 (6 - d))
+// with the three components combined as integers (T1 - T2, T3 - T1 - T2) in
+// two 64-bit words of four and three digit weights, exact until one rounding.  The block then holds the scenario's new voltages, so it
+// decides the stop and, if the scenario goes on, takes a slot of the next
+// sweep and writes the slices of i(v) (or of conj(lambda)) there.  The slot
+// order may differ between runs; no result depends on it.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double exact_double(long long x) {   // |x| < 2^51
+  return __longlong_as_double(x + 0x4338000000000000ll) - 6755399441055744.0;
+}
+
+// hi 2^24 + lo, rounded once: hi's low 24 bits join lo, so both conversions
+// are exact for every size the path takes.
+__device__ __forceinline__ double recombine(long long hi, long long lo) {
+  return fma(exact_double(hi >> 24), 0x1p48, exact_double(((hi & 0xFFFFFFll) << 24) + lo));
+}
+
+template <bool ADJ>
+__device__ __forceinline__ void operand_of_bus(const SolveCtx& c, int b, int n, int j0, int m,
+                                               double inv_s, const double2 (&v)[3],
+                                               double2 (&x)[3]) {
+  const int64_t e = (int64_t)b * n + j0;
+  double2 sw[3], sd[3];
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    sw[p] = (c.S_wye && p < m) ? c.S_wye[e + p] : make_double2(0.0, 0.0);
+    sd[p] = (c.S_del && p < m) ? c.S_del[e + p] : make_double2(0.0, 0.0);
+  }
+  if (!ADJ) {
+    bus_injection_one(v, sw, sd, m, x);
+  } else {
+    double2 vf[3], g[3];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      vf[p] = p < m ? c.Vf[e + p] : make_double2(1.0, 0.0);
+      g[p] = p < m ? c.G[e + p] : make_double2(0.0, 0.0);
+    }
+    adjoint_rhs(vf, v, g, inv_s, sw, sd, m, x);
+  }
+#pragma unroll
+  for (int p = 0; p < 3; ++p)
+    if (p >= m) x[p] = make_double2(0.0, 0.0);
+}
+
+template <bool ADJ, bool FIRST>
+__global__ void __launch_bounds__(256, 2)
+k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs,
+             const double2* __restrict__ w, int n, int K_pad, int64_t rows,
+             cudaGraphConditionalHandle h, int use_handle) {
+  extern __shared__ double2 op[];   // [n] operand of the next sweep
+  __shared__ unsigned long long red[8];
+  __shared__ double sred[8];
+  __shared__ int s_keep, s_slot;
+  const SolveCtx c = *ctx;
+  const int tid = threadIdx.x;
+  const int ld = (n + 7) & ~7;
+  const int nb = (n + 2) / 3;
+  const int par = c.iter & 1;
+  const int32_t* const list = par ? c.list2 : c.list;
+  int32_t* const list_out = FIRST ? nullptr : (par ? c.list : c.list2);
+  const double* const xs = c.xs + (int64_t)par * rows;
+  double* const xs_out = c.xs + (int64_t)(FIRST ? par : par ^ 1) * rows;
+  const int it = c.iter + 1;
+  const bool summag = c.rule == ZBUS_CONV_SUMMAG;
+  for (int slot = blockIdx.x; slot < c.count; slot += gridDim.x) {
+    const int b = list[slot];
+    const bool in = ZB_IN(b, c.B, 0x501u);
+    int out_slot = slot;
+    double2* const V = c.V + (int64_t)(in ? b : 0) * n;
+    unsigned long long top = 0ull;       // largest |Re|, |Im| of the operand
+    unsigned long long st2 = 0ull;       // largest squared step, bit pattern
+    unsigned long long sth = 0ull;       // largest step whose square leaves the range
+    double dsum = 0.0;
+    const double xb = FIRST ? 0.0 : xs[slot];
+    const double inv_s = ADJ ? 1.0 / c.gscale[in ? b : 0] : 0.0;
+    if (in)
+      for (int k = tid; k < nb; k += blockDim.x) {
+        const int j0 = 3 * k, m = min(3, n - j0);
+        double2 v[3];
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+          const int j = j0 + p;
+          v[p] = make_double2(1.0, 0.0);
+          if (p >= m) continue;
+          const double2 vo = V[j];
+          if (FIRST) {
+            v[p] = vo;
+            continue;
+          }
+          const int32_t* D = c.D + (int64_t)slot * ld + j;
+          const int64_t plane = rows * ld;
+          long long hi[3], lo[3];
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            int32_t t[SPLIT_S];
+#pragma unroll
+            for (int d = 0; d < SPLIT_S; ++d) t[d] = D[(q * SPLIT_S + d) * plane];
+            hi[q] = ((long long)t[0] << 24) + ((long long)t[1] << 16) + ((long long)t[2] << 8) +
+                    t[3];
+            lo[q] = ((long long)t[4] << 16) + ((long long)t[5] << 8) + t[6];
+          }
+          const double re = recombine(hi[0] - hi[1], lo[0] - lo[1]);
+          const double im = recombine(hi[2] - hi[0] - hi[1], lo[2] - lo[0] - lo[1]);
+          const double s = zs[j] * xb;
+          const double2 wj = ADJ ? make_double2(0.0, 0.0) : w[j];
+          v[p] = make_double2(fma(re, s, wj.x), fma(im, s, wj.y));
+          V[j] = v[p];
+          const double dx = v[p].x - vo.x, dy = v[p].y - vo.y;
+          const double q2 = fma(dx, dx, dy * dy);
+          const unsigned long long qb = abs_bits(q2);
+          if ((unsigned)(qb >> 52) - 128u < 1792u) {   // far inside the range of squares
+            st2 = max_u64(st2, qb);
+          } else if ((abs_bits(dx) | abs_bits(dy)) != 0ull) {
+            const unsigned long long hb = abs_bits(hypot(dx, dy));
+            sth = max_u64(sth, hb > 0x7FF0000000000000ull ? 0x7FF0000000000000ull : hb);
+          }
+          if (summag) dsum += hypot(v[p].x, v[p].y) - hypot(vo.x, vo.y);
+        }
+        double2 x[3];
+        operand_of_bus<ADJ>(c, b, n, j0, m, inv_s, v, x);
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+          if (p < m) {
+            op[j0 + p] = x[p];
+            top = max_u64(top, max_u64(abs_bits(x[p].x), abs_bits(x[p].y)));
+          }
+      }
+    if (!FIRST) {
+      st2 = block_max_u64(st2, red);
+      sth = block_max_u64(sth, red);
+      if (summag) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
+        if ((tid & 31) == 0) sred[tid >> 5] = dsum;
+        __syncthreads();
+      }
+      if (tid == 0) {
+        double delta = fmax(sqrt(__longlong_as_double((long long)st2)),
+                            __longlong_as_double((long long)sth));
+        if (summag) {
+          double u = 0.0;
+          for (int q = 0; q < (int)(blockDim.x >> 5); ++q) u += sred[q];
+          delta = fabs(u);
+        }
+        int keep = 0;
+        if (in) {
+          c.iters[b] = it;
+          if (!isfinite(delta) || c.err != 0) {
+            c.conv[b] = 0;
+          } else if (delta <= c.tol) {
+            c.conv[b] = 1;
+          } else if (it < c.max_iter) {
+            keep = 1;
+          }
+        }
+        s_keep = keep;
+        if (keep) {
+          const int o = atomicAdd(&ctx->next, 1);
+          list_out[o] = b;
+          s_slot = o;
+        }
+      }
+      __syncthreads();
+      if (!s_keep) {
+        __syncthreads();
+        continue;
+      }
+      out_slot = s_slot;
+    }
+    top = block_max_u64(top, red);
+    // a value that is not finite: the scale carries it to every output
+    const bool bad = top >= 0x7FF0000000000000ull;
+    const int e = bad ? 0 : row_exponent(top);
+    __half* out = reinterpret_cast<__half*>(c.X) + (int64_t)out_slot * K_pad;
+    const int64_t plane = rows * K_pad;
+    if (bad) {
+      write_slices([&](int) { return make_double2(0.0, 0.0); }, n, K_pad, 0, out, plane);
+    } else {
+      write_slices([&](int j) { return op[j]; }, n, K_pad, e, out, plane);
+    }
+    if (tid == 0)
+      xs_out[out_slot] = bad ? __longlong_as_double(0x7FF8000000000000ll) : ldexp(1.0, e - 31);
+    __syncthreads();
+  }
+  if (FIRST) return;
+  // the last block closes the sweep
+  __syncthreads();
+  if (tid == 0) {
+    __threadfence();
+    if (atomicAdd(&ctx->done, 1) == (int)gridDim.x - 1) {
+      __threadfence();
+      const int left = atomicAdd(&ctx->next, 0);
+      if (c.hist && c.iter < c.hist_n) c.hist[c.iter] = c.count;
+      ctx->count = left;
+      ctx->iter = it;
+      ctx->next = 0;
+      ctx->done = 0;
+      if (use_handle) cudaGraphSetConditional(h, left > 0 ? 1u : 0u);
+    }
+  }
+}
+
+PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
+  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+  if (!fn) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
+                                         &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
+  }
+  return fn;
+}
+
+// Planes [21][rows][K_pad] of FP16 as a 3D tensor, boxes of 64 x box_rows;
+// rows past the end read as zero.
+zbus_status make_map(CUtensorMap* map, const void* base, int K_pad, int64_t rows, int box_rows) {
+  auto fn = encode_fn();
+  if (!fn) return fail(ZBUS_ERR_UNSUPPORTED, "cuTensorMapEncodeTiled is not available");
+  cuuint64_t dims[3] = {(cuuint64_t)K_pad, (cuuint64_t)rows, (cuuint64_t)SPLIT_PLANES};
+  cuuint64_t strides[2] = {(cuuint64_t)K_pad * 2, (cuuint64_t)K_pad * 2 * (cuuint64_t)rows};
+  cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)box_rows, 1};
+  cuuint32_t es[3] = {1, 1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, strides,
+                  box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS)
+    return fail(ZBUS_ERR_CUDA, "cuTensorMapEncodeTiled failed with code " + std::to_string((int)r));
+  return ZBUS_OK;
+}
+
+size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
+
+int num_sms() {
+  static int sms = 0;
+  if (!sms) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      sms = 0;
+  }
+  return sms ? sms : 148;
+}
+
+constexpr int STAGES_256 = 4, STAGES_192 = 5;
+template <int BN, int STAGES>
+constexpr size_t gemm_smem() {
+  return (size_t)STAGES * (BM + BN) * BK * 2 + 1024 + (2 * STAGES + 5) * 8 + 16;
+}
+
+template <int BN, int STAGES>
+zbus_status launch_gemm(SolveCtx* ctx, const SplitScratch& s, const SplitOps& ops, int n,
+                        int64_t batch, cudaStream_t st) {
+  constexpr size_t smem = gemm_smem<BN, STAGES>();
+  ZB_CUDA(cudaFuncSetAttribute(k_split_gemm<BN, STAGES>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int64_t items = (int64_t)SPLIT_PLANES * ((batch + BM - 1) / BM) * ((n + BN - 1) / BN);
+  const int grid = (int)std::min<int64_t>(items, num_sms());
+  k_split_gemm<BN, STAGES><<<grid, GEMM_THREADS, smem, st>>>(ctx, s.map, ops.map, n,
+                                                             split_kpad(n) / BK, s.rows);
+  return ZBUS_OK;
+}
+
+int step_threads(int n) { return n <= 3 * 160 ? 128 : 256; }
+
+int step_grid(int64_t batch) {
+  return (int)std::min<int64_t>(batch, (int64_t)num_sms() * 16);
+}
+
+}  // namespace
+
+size_t split_scratch_bytes(int n, int64_t rows) {
+  return a256((size_t)SPLIT_PLANES * rows * split_kpad(n) * 2) +
+         a256((size_t)SPLIT_PLANES * rows * split_ld(n) * 4) + a256((size_t)rows * 2 * 8) +
+         a256((size_t)rows * 4);
+}
+
+zbus_status split_scratch_bind(SplitScratch* s, void* base, int n, int64_t rows) {
+  char* p = (char*)base;
+  s->rows = rows;
+  s->X = p;
+  p += a256((size_t)SPLIT_PLANES * rows * split_kpad(n) * 2);
+  s->D = (int32_t*)p;
+  p += a256((size_t)SPLIT_PLANES * rows * split_ld(n) * 4);
+  s->xs = (double*)p;
+  p += a256((size_t)rows * 2 * 8);
+  s->list2 = (int32_t*)p;
+  return make_map(&s->map, s->X, split_kpad(n), rows, BM);
+}
+
+zbus_status split_pack(SplitOps* ops, const double* Zr, const double* Zi, int n, int n_pad,
+                       cudaStream_t st) {
+  if (ops->Z) return ZBUS_OK;
+  const int K = split_kpad(n);
+  // N-tile: 192 or 256 outputs, whichever leaves less of the last tile idle
+  ops->BN = round_up(n, 192) < round_up(n, 256) ? 192 : 256;
+  zbus_status s = ZBUS_OK;
+  cudaError_t ce;
+  if ((ce = cudaMalloc(&ops->Z, (size_t)SPLIT_PLANES * n * K * 2)) != cudaSuccess ||
+      (ce = cudaMalloc((void**)&ops->zs, (size_t)n * sizeof(double))) != cudaSuccess) {
+    s = cuda_fail(ce, "cudaMalloc(slices of Z)", __FILE__, __LINE__);
+  } else {
+    k_split_pack<<<n, 256, 0, st>>>(Zr, Zi, n, n_pad, K, (__half*)ops->Z, ops->zs);
+    if ((ce = cudaGetLastError()) != cudaSuccess ||
+        (ce = cudaStreamSynchronize(st)) != cudaSuccess)
+      s = cuda_fail(ce, "slices of Z", __FILE__, __LINE__);
+    else
+      s = make_map(&ops->map, ops->Z, K, n, ops->BN);
+  }
+  if (s != ZBUS_OK) split_release(ops);
+  return s;
+}
+
+void split_release(SplitOps* ops) {
+  cudaFree(ops->Z);
+  cudaFree(ops->zs);
+  ops->Z = nullptr;
+  ops->zs = nullptr;
+}
+
+void split_fill_ctx(SolveCtx* h, const SplitScratch& s) {
+  h->X = s.X;
+  h->D = s.D;
+  h->xs = s.xs;
+  h->list2 = s.list2;
+  h->next = 0;
+  h->done = 0;
+}
+
+zbus_status launch_split_gemm(SolveCtx* ctx, const SplitScratch& s, const SplitOps& ops, int n,
+                              int64_t batch, cudaStream_t st) {
+  return ops.BN == 192 ? launch_gemm<192, STAGES_192>(ctx, s, ops, n, batch, st)
+                       : launch_gemm<256, STAGES_256>(ctx, s, ops, n, batch, st);
+}
+
+namespace {
+
+template <bool ADJ, bool FIRST>
+void launch_step(SolveCtx* ctx, const double* zs, const double2* w, int n, int64_t batch,
+                 int64_t rows, cudaGraphConditionalHandle h, bool use_handle, cudaStream_t st) {
+  const size_t smem = (size_t)n * sizeof(double2);
+  if (smem > 32 * 1024)
+    cudaFuncSetAttribute(k_split_step<ADJ, FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
+  k_split_step<ADJ, FIRST><<<step_grid(batch), step_threads(n), smem, st>>>(
+      ctx, zs, w, n, split_kpad(n), rows, h, use_handle ? 1 : 0);
+}
+
+}  // namespace
+
+void launch_split_first(SolveCtx* ctx, int n, int64_t batch, int64_t rows, bool adjoint,
+                        cudaStream_t st) {
+  if (adjoint)
+    launch_step<true, true>(ctx, nullptr, nullptr, n, batch, rows, 0, false, st);
+  else
+    launch_step<false, true>(ctx, nullptr, nullptr, n, batch, rows, 0, false, st);
+}
+
+void launch_split_step(SolveCtx* ctx, const SplitOps& ops, const double2* w, int n, int64_t batch,
+                       int64_t rows, bool adjoint, cudaGraphConditionalHandle h, bool use_handle,
+                       cudaStream_t st) {
+  if (adjoint)
+    launch_step<true, false>(ctx, ops.zs, nullptr, n, batch, rows, h, use_handle, st);
+  else
+    launch_step<false, false>(ctx, ops.zs, w, n, batch, rows, h, use_handle, st);
+}
+
+ZB_CHECK_WORD_ACCESSOR(check_word_split)
+
+}  // namespace zbus

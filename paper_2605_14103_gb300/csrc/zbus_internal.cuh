@@ -92,6 +92,7 @@ uint32_t check_word_group(bool clear);
 uint32_t check_word_adjoint(bool clear);
 uint32_t check_word_nr(bool clear);
 uint32_t check_word_phased(bool clear);
+uint32_t check_word_split(bool clear);
 
 // ---------------------------------------------------------------------------
 // Per-solve device context.  Kernels read pointers and sizes from it, so a
@@ -128,6 +129,34 @@ struct SolveCtx {
   const double2* Vf;      // [B][n]
   const double2* G;       // [B][n]
   const double* gscale;   // [B]
+  // tensor-core contraction of the plain method (split.cu): slices of the
+  // operand, partial products, operand scales and the second active list (the
+  // two alternate with the sweep's parity), the next sweep's count so far and
+  // the blocks that finished this one
+  void* X;
+  int32_t* D;
+  double* xs;
+  int32_t* list2;
+  int32_t next;
+  int32_t done;
+};
+
+// Slices of a matrix for the plain method's tensor-core contraction.
+struct SplitOps {
+  void* Z = nullptr;         // [21][n][K_pad] FP16 digits
+  double* zs = nullptr;      // [n] row scales
+  int BN = 0;                // N-tile
+  CUtensorMap map;           // of Z
+};
+
+// Scratch of `rows` active scenarios, in a caller-provided buffer.
+struct SplitScratch {
+  int64_t rows = 0;
+  void* X = nullptr;         // [21][rows][K_pad] FP16 slices of the operand
+  int32_t* D = nullptr;      // [21][rows][ld] exact partial products
+  double* xs = nullptr;      // [2][rows] operand scales, by sweep parity
+  int32_t* list2 = nullptr;  // [rows] second active list
+  CUtensorMap map;           // of X
 };
 
 struct Workspace {
@@ -288,6 +317,13 @@ struct zbus_network_s {
   int64_t adj_cap = 0;
   double2* adj_tree_scratch = nullptr;   // tree form: [adj_tree_ctas][5 n]
   int64_t adj_tree_ctas = 0;
+  // plain method on the tensor cores: slices of Z and of Z^T (load gradient),
+  // scratch of up to split.rows scenarios
+  zbus::SplitOps split_z;
+  zbus::SplitOps split_zt;
+  zbus::SplitScratch split;
+  void* split_base = nullptr;
+  const zbus::SolveCtx* last_ctx = nullptr;   // context of the last such solve (error word)
 };
 
 namespace zbus {
@@ -341,6 +377,13 @@ void launch_mismatch(const double2* V, const double2* S_wye, const double2* S_de
 
 // api.cu
 zbus_status ensure_workspace(zbus_network net, int64_t B);
+// Whether the plain method of this network runs its contraction on the tensor
+// cores, its operands formed if need be (false: the size is outside that
+// path's range or device memory does not hold them; the FP64 contraction runs)
+bool split_ready(zbus_network net, bool adjoint, cudaStream_t st);
+// Scratch for the split sweeps of up to B scenarios, at most what
+// SPLIT_SCRATCH_MAX holds: the scenarios per pass, 0 if memory does not do
+int64_t split_rows(zbus_network net, int64_t B);
 bool use_graphs();   // false when ZBUS_NO_GRAPH=1 (sweeps launched from the host)
 // One sweep enqueued on a stream: the last kernel sets the WHILE condition
 // through h when use_handle; ev (or nullptr) brackets the kernels.
@@ -349,6 +392,8 @@ typedef zbus_status (*SweepFn)(zbus_network net, int64_t B, int grid,
                                cudaEvent_t* ev);
 // Graph keys besides the precisions of the solve.
 constexpr int32_t GRAPH_KEY_ADJOINT = -2;
+constexpr int32_t GRAPH_KEY_SPLIT = -3;
+constexpr int32_t GRAPH_KEY_SPLIT_ADJOINT = -4;
 zbus_status get_while_graph(zbus_network net, int64_t B, int32_t key, int grid, SweepFn sweep,
                             GraphEntry** out);
 
