@@ -706,9 +706,9 @@ zbus_status solve_device(zbus_network net, int64_t B, const double* S_wye, const
 
   net->last_group = nullptr;
   net->last_ctx = nullptr;   // the sweeps on the CUDA cores have no device-side waits
-  if (o.profile != 1 && B <= F64_BM && net->n_pad <= FUSED_MAX_NPAD) {
-    // a small feeder and at most one tile of scenarios: the whole solve in
-    // one launch (bitwise the results of the sweep-per-launch path below)
+  if (o.profile != 1 && B <= FUSED_MAX_B && net->n_pad <= FUSED_MAX_NPAD) {
+    // a small feeder: the whole solve in one launch, a block per scenario
+    // (bitwise the results of the sweep-per-launch path below)
     launch_solve_fused_f64(net->Zr, net->Zi, net->Zs, net->w, (const double2*)V_init,
                            (const double2*)S_wye, (const double2*)S_delta, net->n, net->n_pad,
                            (int)B, tol, max_iter, o.conv_rule, (double2*)V_out, iters, converged,

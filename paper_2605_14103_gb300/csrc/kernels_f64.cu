@@ -316,8 +316,8 @@ k_gemm3m_f64_small(const SolveCtx* __restrict__ ctx, const double* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------
-// The whole solve of one small feeder in one launch, for the latency case
-// (n_pad <= FUSED_MAX_NPAD unknowns, at most one 32-scenario tile): one block
+// The whole solve of one small feeder in one launch (n_pad <= FUSED_MAX_NPAD
+// unknowns, at most FUSED_MAX_B scenarios): one block
 // per scenario keeps v and the 3M operands in shared memory and runs every
 // sweep (K1, K2, K3) itself, so a solve costs one launch instead of four
 // kernel nodes per sweep.  Every value is formed with the arithmetic of the

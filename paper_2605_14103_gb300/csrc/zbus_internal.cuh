@@ -37,9 +37,13 @@ zbus_status cuda_fail(cudaError_t e, const char* what, const char* file, int lin
 // ---------------------------------------------------------------------------
 constexpr int F64_BM = 32;   // scenarios per tile
 constexpr int F64_BN = 48;   // outputs (16 buses) per tile
-// whole-solve kernel of the latency case: up to 96 padded unknowns, one
-// block of four warps per scenario, batches of one tile at most
+// whole-solve kernel of small feeders: up to 96 padded unknowns, one block of
+// four warps per scenario.  Up to 2048 scenarios: the sweep kernels wait on
+// their launches and on a few long blocks (solves in us, sweeps / whole, 36
+// and 96 unknowns: 64 scenarios 520 / 56 and 1539 / 191, 1024 520 / 247 and
+// 1704 / 950, 4096 576 / 923 and 3193 / 3568, where whole warps pay).
 constexpr int FUSED_MAX_NPAD = 96;
+constexpr int FUSED_MAX_B = 2048;
 constexpr int FUSED_THREADS = 128;
 constexpr int F64_BK = 16;   // k step
 constexpr int F64_PAD = 48;  // n is padded to a multiple of this
@@ -263,6 +267,7 @@ struct zbus_network_s {
   double2* bsr_val = nullptr;   // [nblk][3][3] row-major complex
   int64_t nblk = 0;
   float4* bsr_df = nullptr;     // [nblk][9] double-float copy (mixed sweeps)
+  float* bsr_norm = nullptr;    // [nblk] bound of each block's products (k_block_norm)
   // branches (pairs of identical mirror blocks), for the FP64 test that forms
   // each line's term once: (a, b, block of Y_ab) with a < b, and per block
   // its branch (k, or -(k + 1) for the mirror); nbr = 0 where not available
