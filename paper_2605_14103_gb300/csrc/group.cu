@@ -1503,6 +1503,233 @@ k_check(const double2* __restrict__ V, const double2* __restrict__ Sw,
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same test with its FP64 work left to the buses that need it: the flag
+// only asks whether every |dS_j| is within mtol, and a bus whose mismatch plus
+// a bound of its rounding error is within mtol in a cheaper arithmetic would
+// pass in FP64 too.  Three tiers per bus, from the slots' state (coalesced,
+// one slot per lane), before the slots are admitted again:
+//   FP32          d = v_b - v_a, block products with the hi part of Y, FP32
+//                 currents; error below u (12 + T) (A + 2 I) with u = 2^-24, T
+//                 the bus's blocks, A = sum_t |Y_t|_row max_q |d_q|_1 and I the
+//                 sum of the load currents' magnitudes (products of u: the
+//                 rounding of Y, of d and its terms, of six multiply-adds and
+//                 of the sum over the blocks; 16 u of a current, its FP32 load
+//                 and voltage included, against the 24 u counted);
+//   double-float  error below (4 + T) 2^-40 A, and 4 u I for the FP32 loads;
+//   FP64          check_bus_f64 on the merged voltages and the FP64 loads, as
+//                 k_check, folded into mmax.
+// So a scenario's flag and its selection for correction are those of k_check:
+// mmax is then the largest mismatch of the buses tested in FP64 (0 if none),
+// which is above mtol exactly when the largest of all is.
+//
+// Bound by the latency of the neighbours' state loads, like the FP32 start
+// sweeps: 0.8 ms for 16384 scenarios of 1023 buses against 3.6 for k_branch_f64
+// + k_check, which the FP64 pipe bounds.
+// ---------------------------------------------------------------------------
+constexpr float U32 = 0x1p-24f;
+// Gates from which the tiers pay (whole solve in us, tiers / FP64 test): at
+// 1e-6, the default, 14766 / 17545 (16384 scenarios of 1023 buses, FP16 form)
+// and 821 / 858 (4096 of 127); at 1e-7, where most buses take two tiers, 15751
+// / 17545 and 928 / 858.
+constexpr double SCREEN_MIN_TOL = 5e-7;
+
+// |dS| of a bus from its residual (upper bound of |r_p| in e[p]) and voltages:
+// whether every phase is within mtol (mt2: mtol^2, rounded down).
+__device__ __forceinline__ bool within(const float2* ah, const float2* al, const float* e,
+                                       float mt2) {
+  bool ok = true;
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    const float x = ah[p].x + al[p].x, y = ah[p].y + al[p].y;
+    ok = ok && __fmaf_rn(x, x, y * y) * (e[p] * e[p]) * 1.00001f <= mt2;
+  }
+  return ok;
+}
+
+// Double-float tier of bus a of slot b: true if it passes.
+__device__ __noinline__ bool screen_bus_df(const ItemDesc& it, const float* __restrict__ ynorm,
+                                           int a, int b, float mt2) {
+  const int Bp = it.Bp;
+  float2 ah3[3], al3[3], sw[3], sd[3], inj[3], injl[3];
+  float cur = 0.f, va = 0.f;
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    const int64_t g = (int64_t)(3 * a + p) * Bp + b;
+    ah3[p] = it.Vh[g];
+    al3[p] = it.Vl[g];
+    sw[p] = it.Swf[g];
+    sd[p] = it.Sdf[g];
+    va = fmaxf(va, fabsf(ah3[p].x) + fabsf(ah3[p].y));
+  }
+  bus_injection_f32(ah3, al3, sw, sd, 3, inj, &cur);
+  bus_injection_df(ah3, al3, sw, sd, 3, inj, injl);
+  float ah[3][2], al[3][2];
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    ah[p][0] = -inj[p].x;
+    al[p][0] = -injl[p].x;
+    ah[p][1] = -inj[p].y;
+    al[p][1] = -injl[p].y;
+  }
+  float A = 0.f;
+  for (int t = it.bsr_ptr[a]; t < it.bsr_ptr[a + 1]; ++t) {
+    const int cb = it.bsr_col[t];
+    if (cb >= 0 && !ZB_IN(cb, it.nbus, 0x20du)) continue;
+    float dh[3][2], dl[3][2], dm = 0.f;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      if (cb >= 0) {
+        const int64_t g = (int64_t)(3 * cb + q) * Bp + b;
+        const float2 xh = it.Vh[g], xl = it.Vl[g];
+        df_sub(xh.x, xl.x, ah3[q].x, al3[q].x, dh[q][0], dl[q][0]);
+        df_sub(xh.y, xl.y, ah3[q].y, al3[q].y, dh[q][1], dl[q][1]);
+      } else if (cb == -1) {
+        const float4 s4 = it.vs_df[q];
+        df_sub(s4.x, s4.y, ah3[q].x, al3[q].x, dh[q][0], dl[q][0]);
+        df_sub(s4.z, s4.w, ah3[q].y, al3[q].y, dh[q][1], dl[q][1]);
+      } else {
+        dh[q][0] = ah3[q].x; dl[q][0] = al3[q].x;
+        dh[q][1] = ah3[q].y; dl[q][1] = al3[q].y;
+      }
+      dm = fmaxf(dm, fabsf(dh[q][0]) + fabsf(dh[q][1]));
+    }
+    // the voltages' own last bits count too: d may be far smaller than v
+    A = __fmaf_rn(ynorm[t], __fmaf_rn(0x1p-8f, va, dm), A);
+    const float4* yb = it.bsr_df + (int64_t)t * 9;
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const float4 y = yb[p * 3 + q];
+        df_mac(ah[p][0], al[p][0], y.x, y.y, dh[q][0], dl[q][0]);
+        df_mac(ah[p][0], al[p][0], -y.z, -y.w, dh[q][1], dl[q][1]);
+        df_mac(ah[p][1], al[p][1], y.x, y.y, dh[q][1], dl[q][1]);
+        df_mac(ah[p][1], al[p][1], y.z, y.w, dh[q][0], dl[q][0]);
+      }
+  }
+  const float T = (float)(it.bsr_ptr[a + 1] - it.bsr_ptr[a]);
+  const float err = __fmaf_rn(A, (4.f + T) * 0x1p-40f, cur * (4.f * U32));
+  float e[3];
+#pragma unroll
+  for (int p = 0; p < 3; ++p)
+    e[p] = fabsf(__fadd_rn(ah[p][0], al[p][0])) + fabsf(__fadd_rn(ah[p][1], al[p][1])) + 2.f * err;
+  return within(ah3, al3, e, mt2);
+}
+
+// FP64 tier: the bus's largest |dS|^2, as k_check forms it.
+__device__ __noinline__ unsigned long long screen_bus_f64(
+    const double2* __restrict__ V, const double2* __restrict__ Sw, const double2* __restrict__ Sd,
+    const ItemDesc& it, int a, const double2* __restrict__ bval, const double2* vs3) {
+  const double2 vs[3] = {vs3[0], vs3[1], vs3[2]};
+  return check_bus_f64(V, Sw, Sd, a, it.nbus, it.bsr_ptr, it.bsr_col, bval, vs);
+}
+
+__global__ void __launch_bounds__(32 * CHECK_WARPS, 6)
+k_screen(const ItemDesc* __restrict__ items, int k, int s0, const float* __restrict__ ynorm,
+         float mt2, const double2* __restrict__ V, const double2* __restrict__ Sw64,
+         const double2* __restrict__ Sd64, const uint8_t* __restrict__ conv, int B,
+         const double2* __restrict__ bval64, double2 vs0, double2 vs1, double2 vs2,
+         unsigned long long* __restrict__ mmax, int ny) {
+  const ItemDesc& it = items[k];
+  const int lane = threadIdx.x, ty = threadIdx.y;
+  const int bx = blockIdx.x / ny, by = blockIdx.x % ny;
+  const int bo = bx * 32 + lane;   // scenario of the call
+  const bool live = bo < B && conv[bo] != 0;
+  if (__ballot_sync(0xffffffffu, live) == 0u) return;
+  if (!live) return;
+  const int b = s0 + bo, n = it.n, nb = it.nbus, Bp = it.Bp;
+  const float2* __restrict__ Vh = it.Vh;
+  const float2* __restrict__ Vl = it.Vl;
+  const int32_t* __restrict__ bptr = it.bsr_ptr;
+  const int32_t* __restrict__ bcol = it.bsr_col;
+  const float4* __restrict__ bval = it.bsr_df;
+  unsigned long long worst = 0ull;
+  // runs of CHUNK_BUS buses per warp: neighbours in index often share a line
+  for (int a0 = (by * CHECK_WARPS + ty) * CHUNK_BUS; a0 < nb; a0 += ny * CHECK_WARPS * CHUNK_BUS)
+    for (int a = a0; a < min(nb, a0 + CHUNK_BUS); ++a) {
+      float2 ah3[3], al3[3], sw[3], sd[3], acc[3];
+      float va = 0.f;
+#pragma unroll
+      for (int p = 0; p < 3; ++p) {
+        const int64_t g = (int64_t)(3 * a + p) * Bp + b;
+        ah3[p] = Vh[g];
+        al3[p] = Vl[g];
+        sw[p] = it.Swf[g];
+        sd[p] = it.Sdf[g];
+        va = fmaxf(va, fabsf(ah3[p].x) + fabsf(ah3[p].y));
+      }
+      float cur = 0.f, A = 0.f, mag = 0.f;
+      bus_injection_f32(ah3, al3, sw, sd, 3, acc, &cur);
+#pragma unroll
+      for (int p = 0; p < 3; ++p) acc[p] = make_float2(-acc[p].x, -acc[p].y);
+      const int t0 = bptr[a], t1 = bptr[a + 1];
+      int cb = t0 < t1 ? bcol[t0] : -3;
+      float2 xh[3], xl[3];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) xh[q] = xl[q] = make_float2(0.f, 0.f);
+      if (cb >= 0 && ZB_IN(cb, nb, 0x20eu)) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const int64_t g = (int64_t)(3 * cb + q) * Bp + b;
+          xh[q] = Vh[g];
+          xl[q] = Vl[g];
+        }
+      }
+      for (int t = t0; t < t1; ++t) {
+        const int cn = t + 1 < t1 ? bcol[t + 1] : -3;
+        float2 nh[3], nl[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) nh[q] = nl[q] = make_float2(0.f, 0.f);
+        if (cn >= 0 && ZB_IN(cn, nb, 0x20fu)) {
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            const int64_t g = (int64_t)(3 * cn + q) * Bp + b;
+            nh[q] = Vh[g];
+            nl[q] = Vl[g];
+          }
+        }
+        float2 d[3];
+        float dm = 0.f;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          if (cb >= 0) {
+            d[q] = make_float2((xh[q].x - ah3[q].x) + (xl[q].x - al3[q].x),
+                               (xh[q].y - ah3[q].y) + (xl[q].y - al3[q].y));
+          } else if (cb == -1) {
+            const float4 s4 = it.vs_df[q];
+            d[q] = make_float2((s4.x - ah3[q].x) + (s4.y - al3[q].x),
+                               (s4.z - ah3[q].y) + (s4.w - al3[q].y));
+          } else {
+            d[q] = make_float2(ah3[q].x + al3[q].x, ah3[q].y + al3[q].y);
+          }
+          dm = fmaxf(dm, fabsf(d[q].x) + fabsf(d[q].y));
+        }
+        A = __fmaf_rn(ynorm[t], __fmaf_rn(0x1p-22f, va, dm), A);
+        block_f32(d, bval + (int64_t)t * 9, acc, mag);
+        cb = cn;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          xh[q] = nh[q];
+          xl[q] = nl[q];
+        }
+      }
+      const float err = (float)(12 + t1 - t0) * U32 * (A + 2.f * cur);
+      float e[3];
+#pragma unroll
+      for (int p = 0; p < 3; ++p) e[p] = fabsf(acc[p].x) + fabsf(acc[p].y) + 2.f * err;
+      if (!within(ah3, al3, e, mt2) && !screen_bus_df(it, ynorm, a, b, mt2)) {
+        const int64_t row = (int64_t)bo * n;
+        const double2 vs[3] = {vs0, vs1, vs2};
+        const unsigned long long w =
+            screen_bus_f64(V + row, Sw64 ? Sw64 + row : nullptr, Sd64 ? Sd64 + row : nullptr, it,
+                           a, bval64, vs);
+        worst = w > worst ? w : worst;
+      }
+    }
+  if (worst > 0ull) atomicMax(&mmax[bo], worst);
+}
+
 // Outcome per scenario: mm = sqrt(max |dS|^2); a converged flag with mm above
 // mtol is cleared; mm_out[b] = mm, or -1 for a scenario that was not checked.
 __global__ void k_check_finish(const unsigned long long* mmax, uint8_t* __restrict__ conv, int B,
@@ -2274,18 +2501,26 @@ zbus_status group_collect(Group* g, int k, int64_t s0, int64_t B, double* V_out,
       g->d_items, k, (int)s0, (int)B, (double2*)V_out, iters, converged, mmax);
   int gx = 0, ny = 0;
   check_grid(B, net->n, g->num_sms, &gx, &ny);
-  // branch terms once per line, in the FP64 scratch (free between sweeps)
-  double2* J = nullptr;
-  if (net->nbr > 0 && (size_t)B * net->nbr * 3 * sizeof(double2) <= net->ws.iop_bytes) {
-    J = reinterpret_cast<double2*>(net->ws.Iop);
-    k_branch_f64<<<(unsigned)((int64_t)gx * ny), dim3(32, CHECK_WARPS), 0, st>>>(
-        (const double2*)V_out, converged, (int)B, net->n, net->br_tab, net->nbr, net->bsr_val, J,
-        ny);
+  if (!mm_out && mtol >= SCREEN_MIN_TOL && mtol <= 1e12) {
+    const float mt2 = (float)(mtol * mtol) * 0.9999f;
+    k_screen<<<(unsigned)((int64_t)gx * ny), dim3(32, CHECK_WARPS), 0, st>>>(
+        g->d_items, k, (int)s0, net->bsr_norm, mt2, (const double2*)V_out, (const double2*)S_wye,
+        (const double2*)S_delta, converged, (int)B, net->bsr_val, net->v_slack[0],
+        net->v_slack[1], net->v_slack[2], mmax, ny);
+  } else {
+    // branch terms once per line, in the FP64 scratch (free between sweeps)
+    double2* J = nullptr;
+    if (net->nbr > 0 && (size_t)B * net->nbr * 3 * sizeof(double2) <= net->ws.iop_bytes) {
+      J = reinterpret_cast<double2*>(net->ws.Iop);
+      k_branch_f64<<<(unsigned)((int64_t)gx * ny), dim3(32, CHECK_WARPS), 0, st>>>(
+          (const double2*)V_out, converged, (int)B, net->n, net->br_tab, net->nbr, net->bsr_val,
+          J, ny);
+    }
+    k_check<<<(unsigned)((int64_t)gx * ny), dim3(32, CHECK_WARPS), 0, st>>>(
+        (const double2*)V_out, (const double2*)S_wye, (const double2*)S_delta, converged, (int)B,
+        net->n, net->bsr_ptr, net->bsr_col, net->bsr_val, net->v_slack[0], net->v_slack[1],
+        net->v_slack[2], mmax, ny, J, net->bsr_br, net->nbr);
   }
-  k_check<<<(unsigned)((int64_t)gx * ny), dim3(32, CHECK_WARPS), 0, st>>>(
-      (const double2*)V_out, (const double2*)S_wye, (const double2*)S_delta, converged, (int)B,
-      net->n, net->bsr_ptr, net->bsr_col, net->bsr_val, net->v_slack[0], net->v_slack[1],
-      net->v_slack[2], mmax, ny, J, net->bsr_br, net->nbr);
   if (max_corr <= 0) {
     k_check_finish<<<(unsigned)((B + 255) / 256), 256, 0, st>>>(mmax, converged, (int)B, mtol,
                                                                  mm_out);

@@ -151,7 +151,9 @@ __device__ __forceinline__ void bus_injection_df(const float2* vh, const float2*
 
 // FP32 injection at v = vh + vl rounded to FP32 (rules of bus_injection),
 // for the first sweeps of a cold start, where the residual is still far
-// above the FP32 rounding of the line currents.
+// above the FP32 rounding of the line currents.  cur (if given) gains the
+// magnitudes |Re| + |Im| of every load's current (infinity where a branch
+// voltage is too small beside its phases' to bound the rounding).
 __device__ __forceinline__ float2 load_draw_f32(float2 S, float2 v) {
   if (S.x == 0.f && S.y == 0.f) return make_float2(0.f, 0.f);
   const float inv = __frcp_rn(__fmaf_rn(v.x, v.x, v.y * v.y));
@@ -160,12 +162,16 @@ __device__ __forceinline__ float2 load_draw_f32(float2 S, float2 v) {
 
 __device__ __forceinline__ void bus_injection_f32(const float2* vh, const float2* vl,
                                                   const float2* sw, const float2* sd, int m,
-                                                  float2* inj) {
+                                                  float2* inj, float* cur = nullptr) {
   float2 d[3];
 #pragma unroll
   for (int p = 0; p < 3; ++p)
     d[p] = (p < m && sw) ? load_draw_f32(sw[p], make_float2(vh[p].x + vl[p].x, vh[p].y + vl[p].y))
                          : make_float2(0.f, 0.f);
+  if (cur) {
+#pragma unroll
+    for (int p = 0; p < 3; ++p) *cur += fabsf(d[p].x) + fabsf(d[p].y);
+  }
   if (sd && m == 3) {
     float2 ib[3];   // branches ab, bc, ca
 #pragma unroll
@@ -174,6 +180,13 @@ __device__ __forceinline__ void bus_injection_f32(const float2* vh, const float2
       const float2 u = make_float2((vh[x].x - vh[y].x) + (vl[x].x - vl[y].x),
                                    (vh[x].y - vh[y].y) + (vl[x].y - vl[y].y));
       ib[x] = load_draw_f32(sd[x], u);
+      if (cur) {
+        *cur += fabsf(ib[x].x) + fabsf(ib[x].y);
+        // a branch voltage that cancelled to a few bits: no bound
+        if ((sd[x].x != 0.f || sd[x].y != 0.f) &&
+            fabsf(u.x) + fabsf(u.y) < 0x1p-12f * (fabsf(vh[x].x) + fabsf(vh[x].y)))
+          *cur = __int_as_float(0x7f800000);
+      }
     }
 #pragma unroll
     for (int x = 0; x < 3; ++x) {

@@ -87,6 +87,24 @@ __global__ void k_split_c(const double2* __restrict__ val, int64_t m, float4* ou
   }
 }
 
+// Per branch-form block the largest row sum of max(|Re|, |Im|), rounded up:
+// times the largest |Re d| + |Im d| it bounds the parts of every row of Y d.
+__global__ void k_block_norm(const double2* __restrict__ y, int64_t m, float* __restrict__ out) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    double worst = 0.0;
+    for (int p = 0; p < 3; ++p) {
+      double s = 0.0;
+      for (int q = 0; q < 3; ++q) {
+        const double2 x = y[t * 9 + 3 * p + q];
+        s += fmax(fabs(x.x), fabs(x.y));
+      }
+      worst = fmax(worst, s);
+    }
+    out[t] = __double2float_ru(worst);
+  }
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   if (!fn) {
@@ -127,6 +145,11 @@ zbus_status prepare_df(zbus_network net, cudaStream_t st) {
     const int64_t m = std::max<int64_t>(1, net->nblk * 9);
     ZB_CUDA(cudaMalloc((void**)&net->bsr_df, m * sizeof(float4)));
     ZB_CUDA(cudaMalloc((void**)&net->ys_df, (size_t)net->n * sizeof(float4)));
+    ZB_CUDA(cudaMalloc((void**)&net->bsr_norm,
+                       std::max<int64_t>(1, net->nblk) * sizeof(float)));
+    if (net->nblk > 0)
+      k_block_norm<<<(int)std::min<int64_t>(2048, (net->nblk + 255) / 256), 256, 0, st>>>(
+          net->bsr_val, net->nblk, net->bsr_norm);
     if (net->nblk > 0)
       k_split_c<<<(int)std::min<int64_t>(2048, (net->nblk * 9 + 255) / 256), 256, 0, st>>>(
           net->bsr_val, net->nblk * 9, net->bsr_df);
@@ -194,6 +217,8 @@ void release_mixed_ops(zbus_network net) {
 
 void free_mixed(zbus_network net) {
   cudaFree(net->bsr_df);
+  cudaFree(net->bsr_norm);
+  net->bsr_norm = nullptr;
   cudaFree(net->ys_df);
   cudaFree(net->w_df);
   net->bsr_df = nullptr;
