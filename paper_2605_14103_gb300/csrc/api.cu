@@ -65,7 +65,7 @@ int k_pad_tc(const zbus_network net) { return round_up(2 * net->n, 64); }
 // Scratch of one solve: context, active list, per-tile partials, the FP64
 // contraction operands and the low-precision residual rows.
 struct WsLayout {
-  size_t list, keep, part, iop, R, rinv, mm, vh, vl, swf, sdf, st, amax, mt, sit, sconv, total;
+  size_t list, keep, part, iop, R, rinv, mm, v4, swf, sdf, st, amax, mt, sit, sconv, total;
 };
 
 WsLayout workspace_layout(const zbus_network net, int64_t B) {
@@ -92,10 +92,8 @@ WsLayout workspace_layout(const zbus_network net, int64_t B) {
   L.mm = o;
   o += align256((size_t)B * sizeof(double));
   const size_t f2 = align256(Bp * net->n * sizeof(float2));
-  L.vh = o;
-  o += f2;
-  L.vl = o;
-  o += f2;
+  L.v4 = o;
+  o += 2 * f2;
   L.swf = o;
   o += f2;
   L.sdf = o;
@@ -144,8 +142,7 @@ zbus_status ensure_workspace(zbus_network net, int64_t B) {
   ws.R = (void*)(p + L.R);
   ws.rinv = (float*)(p + L.rinv);
   ws.mm = (double*)(p + L.mm);
-  ws.Vh = (float2*)(p + L.vh);
-  ws.Vl = (float2*)(p + L.vl);
+  ws.V4 = (float4*)(p + L.v4);
   ws.Swf = (float2*)(p + L.swf);
   ws.Sdf = (float2*)(p + L.sdf);
   ws.st = (uint8_t*)(p + L.st);

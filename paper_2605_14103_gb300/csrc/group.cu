@@ -102,17 +102,15 @@ __global__ void k_slot_init(GroupState* __restrict__ gs, const ItemDesc* __restr
   for (int r = ty; r < 32; r += 8) {
     const int j = j0 + r, b = b0 + tx;
     if (j < n && b < B) {
-      const int64_t g = (int64_t)j * Bp + s0 + b;
+      const int64_t g = slot_base(n, s0 + b) + SLOT_BLOCK * j;
       if (WARM) {
         const double2 v = tv[tx][r];
         const float2 xr = df_split(v.x), xi = df_split(v.y);
-        it.Vh[g] = make_float2(xr.x, xi.x);
-        it.Vl[g] = make_float2(xr.y, xi.y);
+        it.V4[g] = make_float4(xr.x, xi.x, xr.y, xi.y);
       } else {
         // no-load start: the double-float copy of w made at setup
         const float4 wd = w_df[j];
-        it.Vh[g] = make_float2(wd.x, wd.z);
-        it.Vl[g] = make_float2(wd.y, wd.w);
+        it.V4[g] = make_float4(wd.x, wd.z, wd.y, wd.w);
       }
       it.Swf[g] = make_float2(d2f_rn(tw[tx][r].x), d2f_rn(tw[tx][r].y));
       it.Sdf[g] = make_float2(d2f_rn(td[tx][r].x), d2f_rn(td[tx][r].y));
@@ -230,10 +228,10 @@ k_residual_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
     c = ldexpf(1.f, e);
     if (ys == 0 && warp == 0) it.rinv[b] = ldexpf(1.f, -e);
   }
-  const float2* __restrict__ Vh = it.Vh;
-  const float2* __restrict__ Vl = it.Vl;
-  const float2* __restrict__ Sw = it.Swf;
-  const float2* __restrict__ Sd = it.Sdf;
+  const int64_t base = slot_base(it.n, b);
+  const float4* __restrict__ V4 = it.V4 + base;
+  const float2* __restrict__ Sw = it.Swf + base;
+  const float2* __restrict__ Sd = it.Sdf + base;
   const int32_t* __restrict__ bptr = it.bsr_ptr;
   const int32_t* __restrict__ bcol = it.bsr_col;
   const float4* __restrict__ bval = it.bsr_df;
@@ -249,9 +247,10 @@ k_residual_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
         float2 ah3[3], al3[3], sw[3], sd[3], inj[3], injl[3];   // own state, loads
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
-          const int64_t g = (int64_t)(3 * a + p) * Bp + b;
-          ah3[p] = Vh[g];
-          al3[p] = Vl[g];
+          const int g = SLOT_BLOCK * (3 * a + p);
+          const float4 v = V4[g];
+          ah3[p] = make_float2(v.x, v.y);
+          al3[p] = make_float2(v.z, v.w);
           sw[p] = Sw[g];
           sd[p] = Sd[g];
         }
@@ -277,9 +276,9 @@ k_residual_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
           if (cb >= 0 && ZB_IN(cb, nb, 0x202u)) {
 #pragma unroll
             for (int q2 = 0; q2 < 3; ++q2) {
-              const int64_t g = (int64_t)(3 * cb + q2) * Bp + b;
-              xh[q2] = Vh[g];
-              xl[q2] = Vl[g];
+              const float4 v = V4[SLOT_BLOCK * (3 * cb + q2)];
+              xh[q2] = make_float2(v.x, v.y);
+              xl[q2] = make_float2(v.z, v.w);
             }
           }
           for (; t < t1; ++t) {
@@ -290,9 +289,9 @@ k_residual_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
             if (cn >= 0 && ZB_IN(cn, nb, 0x203u)) {
 #pragma unroll
               for (int q2 = 0; q2 < 3; ++q2) {
-                const int64_t g = (int64_t)(3 * cn + q2) * Bp + b;
-                nh[q2] = Vh[g];
-                nl[q2] = Vl[g];
+                const float4 v = V4[SLOT_BLOCK * (3 * cn + q2)];
+                nh[q2] = make_float2(v.x, v.y);
+                nl[q2] = make_float2(v.z, v.w);
               }
             }
             if (cb >= 0 && !ZB_IN(cb, nb, 0x204u)) cb = -3;
@@ -346,10 +345,9 @@ k_residual_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
           if (cb >= 0) {
 #pragma unroll
             for (int q2 = 0; q2 < 3; ++q2) {
-              const int64_t g = (int64_t)(3 * cb + q2) * Bp + b;
-              const float2 xh = Vh[g], xl = Vl[g];
-              df_sub(xh.x, xl.x, ah3[q2].x, al3[q2].x, dh[q2][0], dl[q2][0]);
-              df_sub(xh.y, xl.y, ah3[q2].y, al3[q2].y, dh[q2][1], dl[q2][1]);
+              const float4 v = V4[SLOT_BLOCK * (3 * cb + q2)];
+              df_sub(v.x, v.z, ah3[q2].x, al3[q2].x, dh[q2][0], dl[q2][0]);
+              df_sub(v.y, v.w, ah3[q2].y, al3[q2].y, dh[q2][1], dl[q2][1]);
             }
           } else if (cb == -1) {
 #pragma unroll
@@ -390,7 +388,7 @@ k_residual_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
       if constexpr (OUT == RES_F32) {
         if (a < nb && act) {
 #pragma unroll
-          for (int p = 0; p < 3; ++p) it.Rt[(int64_t)(3 * a + p) * Bp + b] = r[p];
+          for (int p = 0; p < 3; ++p) it.Rt[base + SLOT_BLOCK * (3 * a + p)] = r[p];
         }
       } else {
 #pragma unroll
@@ -453,8 +451,10 @@ k_residual_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
 // over K_pad of its item in steps of 64 (128-byte swizzled rows staged by
 // TMA).  Two tensor-memory accumulators (2 x BN columns) let the epilogue of
 // one tile overlap the MMAs of the next.  Warp roles: 0 = TMA producer,
-// 1 = TMEM owner and MMA issuer, 2..5 = epilogue (warp w reads TMEM lanes
-// 32 (w % 4) .. + 31).  Barriers: full / empty per stage (TMA -> MMA -> TMA),
+// 1 = TMEM owner and MMA issuer, 2..9 = epilogue (warp w reads TMEM lanes
+// 32 (w % 4) .. + 31 of one half of the columns: with four warps the state
+// loads and stores of a small feeder's tile took longer than its MMAs, 33
+// against 23 us a sweep at 4096 scenarios of 127 buses).  Barriers: full / empty per stage (TMA -> MMA -> TMA),
 // tfull / tempty per accumulator (MMA -> epilogue -> MMA).
 //
 // L2: every CTA re-reads Z_emb (75 MB at 3069 unknowns) during the launch,
@@ -491,6 +491,8 @@ k_contract_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
   constexpr int A_BYTES = BM * BK * 2;
   constexpr int B_BYTES = BN * BK * 2;
   constexpr int STAGE_BYTES = A_BYTES + ZP * B_BYTES;
+  constexpr int HN = BN / 2;   // columns of one epilogue warp, EC at a time
+  constexpr int EC = 16;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(smem + STAGES * STAGE_BYTES);
@@ -513,7 +515,7 @@ k_contract_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
     }
     for (int u = 0; u < 2; ++u) {
       mbar_init(&tfull[u], 1);
-      mbar_init(&tempty[u], 4);
+      mbar_init(&tempty[u], TC_EPI_WARPS);
     }
     mbar_init(drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -618,7 +620,7 @@ k_contract_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
       }
     }
   } else {
-    const int q = warp & 3;
+    const int q = warp & 3, half = (warp - 2) >> 2;
     const int row = q * 32 + lane;
     const bool summag = gs->rule == ZBUS_CONV_SUMMAG;
     // evict-first for a state larger than L2 keeps, else the default
@@ -636,33 +638,30 @@ k_contract_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
         if (lane == 0) atomicCAS(&gs->err, 0, 103);
         break;
       }
-      const int n = it.n, Bp = it.Bp, ntn = it.ntn;
+      const int n = it.n;
       const int b = mt * BM + row;
       const bool valid = it.st[b] == SLOT_ACTIVE;
       const float rs = valid ? it.rinv[b] : 0.f;
       const float* __restrict__ zinv = it.zinv;
-      float2* __restrict__ Vh = it.Vh + b;
-      float2* __restrict__ Vl = it.Vl + b;
+      float4* __restrict__ V4 = it.V4 + slot_base(n, b);
       float dmax = 0.f, dsum = 0.f;
 #pragma unroll 1
-      for (int c = 0; c < BN / 32; ++c) {
-        const int i0 = (nt * BN + c * 32) >> 1;
-        // the chunk's 16 state entries are requested before any of them is
+      for (int c = 0; c < HN / EC; ++c) {
+        const int i0 = (nt * BN + half * HN + c * EC) >> 1;
+        // the chunk's state entries are requested before any of them is
         // used, so their memory latencies overlap
-        float2 h[16], l[16];
-        float zs[16];
+        float4 vo[EC / 2];
+        float zs[EC / 2];
 #pragma unroll
-        for (int t = 0; t < 16; ++t) {
+        for (int t = 0; t < EC / 2; ++t) {
           const int oi = i0 + t;
           const bool in = valid && oi < n;
-          const int64_t gi = (int64_t)(in ? oi : 0) * Bp;
-          h[t] = in ? ld_f2_hint(Vh + gi, spol) : make_float2(0.f, 0.f);
-          l[t] = in ? ld_f2_hint(Vl + gi, spol) : make_float2(0.f, 0.f);
+          vo[t] = in ? ld_f4_hint(V4 + SLOT_BLOCK * oi, spol) : make_float4(0.f, 0.f, 0.f, 0.f);
           zs[t] = in ? zinv[oi] : 0.f;
         }
-        float v[32];
-        tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + c * 32), v);
-        if (c == BN / 32 - 1) {
+        float v[EC];
+        tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + half * HN + c * EC), v);
+        if (c == HN / EC - 1) {
           // the accumulator is in registers now: hand the buffer back
           tc_fence_before();
           __syncwarp();
@@ -670,28 +669,26 @@ k_contract_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
         }
         if (valid) {
 #pragma unroll
-          for (int t = 0; t < 16; ++t) {
+          for (int t = 0; t < EC / 2; ++t) {
             const int oi = i0 + t;
             if (oi < n) {
               const float sc = rs * zs[t];
               const float dr = v[2 * t] * sc, di = v[2 * t + 1] * sc;
               float sr, er, si, ei;
-              two_sum(h[t].x, dr, sr, er);
-              two_sum(h[t].y, di, si, ei);
+              two_sum(vo[t].x, dr, sr, er);
+              two_sum(vo[t].y, di, si, ei);
               float2 nh, nl;
-              fast_two_sum(sr, __fadd_rn(er, l[t].x), nh.x, nl.x);
-              fast_two_sum(si, __fadd_rn(ei, l[t].y), nh.y, nl.y);
-              const int64_t gi = (int64_t)oi * Bp;
-              st_f2_hint(Vh + gi, nh, spol);
-              st_f2_hint(Vl + gi, nl, spol);
+              fast_two_sum(sr, __fadd_rn(er, vo[t].z), nh.x, nl.x);
+              fast_two_sum(si, __fadd_rn(ei, vo[t].w), nh.y, nl.y);
+              st_f4_hint(V4 + SLOT_BLOCK * oi, make_float4(nh.x, nh.y, nl.x, nl.y), spol);
               float step = sqrtf(__fmaf_rn(dr, dr, di * di));
               if (step != step) step = __int_as_float(0x7f800000);
               dmax = fmaxf(dmax, step);
               if (summag) {
                 // |v + d| - |v| = (2 Re(conj(v) d) + |d|^2) / (|v + d| + |v|)
-                const float o2 = __fmaf_rn(h[t].x, h[t].x, h[t].y * h[t].y);
+                const float o2 = __fmaf_rn(vo[t].x, vo[t].x, vo[t].y * vo[t].y);
                 const float n2 = __fmaf_rn(nh.x, nh.x, nh.y * nh.y);
-                dsum += (2.f * (h[t].x * dr + h[t].y * di) + dr * dr + di * di) /
+                dsum += (2.f * (vo[t].x * dr + vo[t].y * di) + dr * dr + di * di) /
                         (sqrtf(n2) + sqrtf(o2));
               }
             }
@@ -699,8 +696,7 @@ k_contract_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
         }
       }
       if (valid) {
-        it.part[((int64_t)b * ntn + nt) * 2 + 0] = (double)dmax;
-        it.part[((int64_t)b * ntn + nt) * 2 + 1] = (double)dsum;
+        it.part[(int64_t)(2 * nt + half) * it.Bp + b] = make_float2(dmax, dsum);
       }
     }
   }
@@ -724,14 +720,24 @@ __device__ __forceinline__ void decide_slot(const GroupState* __restrict__ gs, c
   if (b < it.Bp && it.st[b] == SLOT_ACTIVE) {
     const int sw = it.it[b] + 1;
     it.it[b] = sw;
-    const int ntn = it.ntn;
-    const double* part = it.part + (int64_t)b * ntn * 2;
-    double dmax = 0.0, dsum = 0.0;
-    for (int t = 0; t < ntn; ++t) {
-      dmax = fmax(dmax, part[2 * t]);
-      dsum += part[2 * t + 1];
+    const float2* part = it.part + b;
+    const int np = 2 * it.ntn;
+    const bool summag = gs->rule == ZBUS_CONV_SUMMAG;
+    float dmax = 0.f;
+    double dsum = 0.0;
+    // 16 requests in flight; the sum's order is that of the tiles
+    for (int t0 = 0; t0 < np; t0 += 16) {
+      float2 x[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u)
+        x[u] = t0 + u < np ? part[(int64_t)(t0 + u) * it.Bp] : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        dmax = fmaxf(dmax, x[u].x);
+        if (summag) dsum += (double)x[u].y;
+      }
     }
-    const double delta = gs->rule == ZBUS_CONV_SUMMAG ? fabs(dsum) : dmax;
+    const double delta = summag ? fabs(dsum) : (double)dmax;
     // a sweep on the FP32 residual never stops a slot
     const bool lp = it.amax[3 * it.Bp + b] != 0.f;
     if (!isfinite(delta)) {
@@ -818,7 +824,8 @@ k_tree_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items,
     if (threadIdx.x == 0) tree_block_done(gs, 0, h, use_handle);
     return;
   }
-  const int Bp = it.Bp, D = it.tlevels, nb = it.nbus;
+  const int D = it.tlevels, nb = it.nbus;
+  const int64_t base = slot_base(it.n, b);
   int4* node = reinterpret_cast<int4*>(tsm);                 // bus, parent, children
   __half2* zt = reinterpret_cast<__half2*>(node + nb);       // [nb][9]
   float* zst = reinterpret_cast<float*>(zt + 9 * nb);        // [nb]
@@ -844,7 +851,7 @@ k_tree_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items,
   // memory, or (ONCHIP, small feeders) a shared-memory copy of the block's
   // 32 slots, so that the level sweeps never leave the SM
   float2* R;
-  int64_t rs;
+  constexpr int rs = ONCHIP ? 32 : SLOT_BLOCK;
   if (ONCHIP) {
     float2* rsm = reinterpret_cast<float2*>(tsm + tree_table_bytes(nb));
     const int n = 3 * nb;
@@ -853,7 +860,7 @@ k_tree_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items,
 #pragma unroll
       for (int u = 0; u < TREE_BATCH; ++u) {
         const int j = j0 + u * TREE_WARPS;
-        v[u] = (act && j < n) ? it.Rt[(int64_t)j * Bp + b] : make_float2(0.f, 0.f);
+        v[u] = (act && j < n) ? it.Rt[base + SLOT_BLOCK * j] : make_float2(0.f, 0.f);
       }
 #pragma unroll
       for (int u = 0; u < TREE_BATCH; ++u) {
@@ -863,12 +870,10 @@ k_tree_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items,
     }
     __syncthreads();
     R = rsm + lane;
-    rs = 32;
   } else {
-    R = it.Rt + b;
-    rs = Bp;
+    R = it.Rt + base;
   }
-  const int64_t r3 = 3 * rs;
+  constexpr int r3 = 3 * rs;
   const int first = warp;   // the warp's first bus of a level
   constexpr int STRIDE = TREE_WARPS;
   for (int L = D - 2; L >= 0; --L) {
@@ -966,17 +971,16 @@ k_tree_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items,
   float dmax = 0.f, dsum = 0.f;
   if (act) {
     for (int a0 = first; a0 < nb; a0 += STRIDE * TREE_BATCH) {
-      float2 xb[TREE_BATCH][3], hb[TREE_BATCH][3], lb[TREE_BATCH][3];
+      float2 xb[TREE_BATCH][3];
+      float4 vb[TREE_BATCH][3];
 #pragma unroll
       for (int u = 0; u < TREE_BATCH; ++u) {
         const int a = a0 + u * STRIDE;
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
           const int j = 3 * (a < nb ? a : 0) + p;
-          const int64_t g = (int64_t)j * Bp + b;
           xb[u][p] = R[j * rs];
-          hb[u][p] = it.Vh[g];
-          lb[u][p] = it.Vl[g];
+          vb[u][p] = it.V4[base + SLOT_BLOCK * j];
         }
       }
 #pragma unroll
@@ -985,16 +989,15 @@ k_tree_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items,
         if (a >= nb) break;
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
-          const float2 d = xb[u][p], h = hb[u][p], l = lb[u][p];
+          const float2 d = xb[u][p];
+          const float4 h = vb[u][p];
           float sr, er, si, ei;
           two_sum(h.x, d.x, sr, er);
           two_sum(h.y, d.y, si, ei);
           float2 nh, nl;
-          fast_two_sum(sr, __fadd_rn(er, l.x), nh.x, nl.x);
-          fast_two_sum(si, __fadd_rn(ei, l.y), nh.y, nl.y);
-          const int64_t g = (int64_t)(3 * a + p) * Bp + b;
-          it.Vh[g] = nh;
-          it.Vl[g] = nl;
+          fast_two_sum(sr, __fadd_rn(er, h.z), nh.x, nl.x);
+          fast_two_sum(si, __fadd_rn(ei, h.w), nh.y, nl.y);
+          it.V4[base + SLOT_BLOCK * (3 * a + p)] = make_float4(nh.x, nh.y, nl.x, nl.y);
           float step = sqrtf(__fmaf_rn(d.x, d.x, d.y * d.y));
           if (step != step) step = __int_as_float(0x7f800000);
           dmax = fmaxf(dmax, step);
@@ -1194,24 +1197,19 @@ k_slot_merge(const ItemDesc* __restrict__ items, int k, int s0, int B,
              uint8_t* __restrict__ conv, unsigned long long* __restrict__ mmax) {
   extern __shared__ double2 tm[];   // [MERGE_T slots][MERGE_T + 1 unknowns]
   const ItemDesc it = items[k];
-  const int n = it.n, Bp = it.Bp;
+  const int n = it.n;
   const int j0 = blockIdx.x * MERGE_T, b0 = blockIdx.y * MERGE_T;
   const int tx = threadIdx.x, ty = threadIdx.y;
-  const float2* __restrict__ Vh = it.Vh;
-  const float2* __restrict__ Vl = it.Vl;
-  float2 h[8][2], l[8][2];
+  const float4* __restrict__ V4 = it.V4;
+  float4 v[8][2];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int j = j0 + ty + 8 * i;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       const int b = b0 + tx + 32 * c;
-      h[i][c] = l[i][c] = make_float2(0.f, 0.f);
-      if (j < n && b < B) {
-        const int64_t g = (int64_t)j * Bp + s0 + b;
-        h[i][c] = Vh[g];
-        l[i][c] = Vl[g];
-      }
+      v[i][c] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (j < n && b < B) v[i][c] = V4[slot_base(n, s0 + b) + SLOT_BLOCK * j];
     }
   }
 #pragma unroll
@@ -1219,8 +1217,8 @@ k_slot_merge(const ItemDesc* __restrict__ items, int k, int s0, int B,
 #pragma unroll
     for (int c = 0; c < 2; ++c)
       tm[(tx + 32 * c) * (MERGE_T + 1) + ty + 8 * i] =
-          make_double2(f2d_exact(h[i][c].x) + f2d_exact(l[i][c].x),
-                       f2d_exact(h[i][c].y) + f2d_exact(l[i][c].y));
+          make_double2(f2d_exact(v[i][c].x) + f2d_exact(v[i][c].z),
+                       f2d_exact(v[i][c].y) + f2d_exact(v[i][c].w));
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -1550,16 +1548,18 @@ __device__ __forceinline__ bool within(const float2* ah, const float2* al, const
 // Double-float tier of bus a of slot b: true if it passes.
 __device__ __noinline__ bool screen_bus_df(const ItemDesc& it, const float* __restrict__ ynorm,
                                            int a, int b, float mt2) {
-  const int Bp = it.Bp;
+  const int64_t base = slot_base(it.n, b);
+  const float4* __restrict__ V4 = it.V4 + base;
   float2 ah3[3], al3[3], sw[3], sd[3], inj[3], injl[3];
   float cur = 0.f, va = 0.f;
 #pragma unroll
   for (int p = 0; p < 3; ++p) {
-    const int64_t g = (int64_t)(3 * a + p) * Bp + b;
-    ah3[p] = it.Vh[g];
-    al3[p] = it.Vl[g];
-    sw[p] = it.Swf[g];
-    sd[p] = it.Sdf[g];
+    const int g = SLOT_BLOCK * (3 * a + p);
+    const float4 v = V4[g];
+    ah3[p] = make_float2(v.x, v.y);
+    al3[p] = make_float2(v.z, v.w);
+    sw[p] = it.Swf[base + g];
+    sd[p] = it.Sdf[base + g];
     va = fmaxf(va, fabsf(ah3[p].x) + fabsf(ah3[p].y));
   }
   bus_injection_f32(ah3, al3, sw, sd, 3, inj, &cur);
@@ -1580,10 +1580,9 @@ __device__ __noinline__ bool screen_bus_df(const ItemDesc& it, const float* __re
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
       if (cb >= 0) {
-        const int64_t g = (int64_t)(3 * cb + q) * Bp + b;
-        const float2 xh = it.Vh[g], xl = it.Vl[g];
-        df_sub(xh.x, xl.x, ah3[q].x, al3[q].x, dh[q][0], dl[q][0]);
-        df_sub(xh.y, xl.y, ah3[q].y, al3[q].y, dh[q][1], dl[q][1]);
+        const float4 v = V4[SLOT_BLOCK * (3 * cb + q)];
+        df_sub(v.x, v.z, ah3[q].x, al3[q].x, dh[q][0], dl[q][0]);
+        df_sub(v.y, v.w, ah3[q].y, al3[q].y, dh[q][1], dl[q][1]);
       } else if (cb == -1) {
         const float4 s4 = it.vs_df[q];
         df_sub(s4.x, s4.y, ah3[q].x, al3[q].x, dh[q][0], dl[q][0]);
@@ -1638,9 +1637,11 @@ k_screen(const ItemDesc* __restrict__ items, int k, int s0, const float* __restr
   const bool live = bo < B && conv[bo] != 0;
   if (__ballot_sync(0xffffffffu, live) == 0u) return;
   if (!live) return;
-  const int b = s0 + bo, n = it.n, nb = it.nbus, Bp = it.Bp;
-  const float2* __restrict__ Vh = it.Vh;
-  const float2* __restrict__ Vl = it.Vl;
+  const int b = s0 + bo, n = it.n, nb = it.nbus;
+  const int64_t base = slot_base(n, b);
+  const float4* __restrict__ V4 = it.V4 + base;
+  const float2* __restrict__ Sw = it.Swf + base;
+  const float2* __restrict__ Sd = it.Sdf + base;
   const int32_t* __restrict__ bptr = it.bsr_ptr;
   const int32_t* __restrict__ bcol = it.bsr_col;
   const float4* __restrict__ bval = it.bsr_df;
@@ -1652,11 +1653,12 @@ k_screen(const ItemDesc* __restrict__ items, int k, int s0, const float* __restr
       float va = 0.f;
 #pragma unroll
       for (int p = 0; p < 3; ++p) {
-        const int64_t g = (int64_t)(3 * a + p) * Bp + b;
-        ah3[p] = Vh[g];
-        al3[p] = Vl[g];
-        sw[p] = it.Swf[g];
-        sd[p] = it.Sdf[g];
+        const int g = SLOT_BLOCK * (3 * a + p);
+        const float4 v = V4[g];
+        ah3[p] = make_float2(v.x, v.y);
+        al3[p] = make_float2(v.z, v.w);
+        sw[p] = Sw[g];
+        sd[p] = Sd[g];
         va = fmaxf(va, fabsf(ah3[p].x) + fabsf(ah3[p].y));
       }
       float cur = 0.f, A = 0.f, mag = 0.f;
@@ -1671,9 +1673,9 @@ k_screen(const ItemDesc* __restrict__ items, int k, int s0, const float* __restr
       if (cb >= 0 && ZB_IN(cb, nb, 0x20eu)) {
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-          const int64_t g = (int64_t)(3 * cb + q) * Bp + b;
-          xh[q] = Vh[g];
-          xl[q] = Vl[g];
+          const float4 v = V4[SLOT_BLOCK * (3 * cb + q)];
+          xh[q] = make_float2(v.x, v.y);
+          xl[q] = make_float2(v.z, v.w);
         }
       }
       for (int t = t0; t < t1; ++t) {
@@ -1684,9 +1686,9 @@ k_screen(const ItemDesc* __restrict__ items, int k, int s0, const float* __restr
         if (cn >= 0 && ZB_IN(cn, nb, 0x20fu)) {
 #pragma unroll
           for (int q = 0; q < 3; ++q) {
-            const int64_t g = (int64_t)(3 * cn + q) * Bp + b;
-            nh[q] = Vh[g];
-            nl[q] = Vl[g];
+            const float4 v = V4[SLOT_BLOCK * (3 * cn + q)];
+            nh[q] = make_float2(v.x, v.y);
+            nl[q] = make_float2(v.z, v.w);
           }
         }
         float2 d[3];
@@ -2127,8 +2129,7 @@ zbus_status group_build(Group* g, const std::vector<zbus_network>& nets,
       d.N_pad = round_up(2 * net->n, 256);
       d.ntn = d.N_pad / g->BN;
     }
-    d.Vh = ws.Vh;
-    d.Vl = ws.Vl;
+    d.V4 = ws.V4;
     d.Swf = ws.Swf;
     d.Sdf = ws.Sdf;
     d.st = ws.st;
@@ -2137,7 +2138,7 @@ zbus_status group_build(Group* g, const std::vector<zbus_network>& nets,
     d.amax = ws.amax;
     d.R = ws.R;
     d.rinv = ws.rinv;
-    d.part = ws.part;
+    d.part = reinterpret_cast<float2*>(ws.part);
     const int rows_pad = tree ? d.n : d.K_pad / 2;
     const int nchunks = (rows_pad + CHUNK_ROWS - 1) / CHUNK_ROWS;
     d.res_split = (nchunks + RES_WARPS - 1) / RES_WARPS;

@@ -19,6 +19,19 @@ constexpr uint8_t SLOT_ACTIVE = 0;
 constexpr uint8_t SLOT_DONE = 1;   // stopped, result not yet collected
 constexpr uint8_t SLOT_FREE = 2;
 
+// Slot state layout: the 128 slots of a contraction tile are one block of
+// memory, unknown by unknown, so a warp's 32 slots stay coalesced while the
+// state that a tile or a residual block walks over is one run of a few MB
+// instead of one row piece every 8 Bp bytes, and an unknown's hi and lo parts
+// are one 16-byte access.  At 16384 scenarios of 1023 buses a residual sweep
+// went from 760 to 717 us (FP16) and 697 to 661 (tree), the tree sweep from
+// 732 to 714.
+constexpr int SLOT_BLOCK = 128;
+// Index of slot b's unknown 0; unknown j is SLOT_BLOCK * j further.
+__host__ __device__ __forceinline__ int64_t slot_base(int n, int b) {
+  return (int64_t)((unsigned)b / SLOT_BLOCK) * n * SLOT_BLOCK + (unsigned)b % SLOT_BLOCK;
+}
+
 // One feeder of a group (device-visible).
 struct ItemDesc {
   // network operands
@@ -29,9 +42,8 @@ struct ItemDesc {
   const float* zinv;        // [N_pad / 2] inverse row scales of Z
   int32_t n, nbus, K_pad, N_pad, ntn;
   int32_t Bp;               // slot capacity, multiple of 128
-  // slot state, scenario-minor [n][Bp]
-  float2* Vh;
-  float2* Vl;
+  // slot state in blocks of 128 slots, [Bp / 128][n][128] (slot_base)
+  float4* V4;               // voltage, double-float: hi (re, im), lo (re, im)
   float2* Swf;              // FP32 wye loads (zeros where absent)
   float2* Sdf;              // FP32 delta loads (zeros where absent)
   uint8_t* st;              // [Bp] SLOT_*
@@ -42,14 +54,15 @@ struct ItemDesc {
                             // sweeps), the FP32-sweep flag (nonzero: on)
   void* R;                  // [Bp][K_pad] fp16 / bf16 residual rows
   float* rinv;              // [Bp] inverse residual scales
-  double* part;             // [Bp][ntn][2] per-tile step partials
+  float2* part;             // [2 ntn][Bp] step partials (max, sum-of-magnitudes change)
+                            // per half N-tile
   // tree sweep (ZBUS_TREE_SWEEP): radial structure and FP32 residual
   const int4* t_node;       // [nbus] per breadth-first position: bus, parent, children range
   const int32_t* t_lvl;     // [tlevels + 1] level ranges of positions
   const uint8_t* t_mask;    // [nbus] phases of each position's parent line
   const float2* t_z;        // [nbus][9] scaled parent-branch impedances
   const float* t_zs;        // [nbus] their scales
-  float2* Rt;               // [n][Bp] FP32 residual, scenario-minor
+  float2* Rt;               // FP32 residual, in the slot state's layout
   int32_t tlevels;          // depth of the tree + 1
   int32_t tree_begin;       // first tree block of this item
   // launch decomposition

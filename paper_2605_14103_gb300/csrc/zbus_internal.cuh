@@ -176,10 +176,9 @@ struct Workspace {
   float* rinv = nullptr;     // mixed: [cap_B] inverse residual scales
   double* mm = nullptr;      // mixed: [cap_B] final FP64 mismatch (-1 if not checked)
   uint8_t* keep = nullptr;   // [cap_B]
-  float2* Vh = nullptr;      // mixed: [n][cap_Bp] double-float state, hi
-  float2* Vl = nullptr;      // mixed: [n][cap_Bp] lo
-  float2* Swf = nullptr;     // mixed: [n][cap_Bp] FP32 wye loads
-  float2* Sdf = nullptr;     // mixed: [n][cap_Bp] FP32 delta loads
+  float4* V4 = nullptr;      // mixed: double-float state (slot layout, group.cuh)
+  float2* Swf = nullptr;     // mixed: FP32 wye loads (the same layout)
+  float2* Sdf = nullptr;     // mixed: FP32 delta loads
   uint8_t* st = nullptr;     // mixed: [cap_Bp]
   float* amax = nullptr;     // mixed: [2][cap_Bp]
   int32_t* mt = nullptr;     // mixed: [2][cap_Bp / 128] tile list and flags
