@@ -62,6 +62,43 @@ void cache_evict(zbus_network net) {
   release_z(net);
 }
 
+// Slot states of every feeder ([n_items][cap] bytes, cap a multiple of 128)
+// and the device error word into pinned host memory: one launch a sweep in
+// the place of a copy per feeder.
+__global__ void k_serve_status(const ItemDesc* __restrict__ items, int n_items, int64_t cap,
+                               const int32_t* __restrict__ err, uint8_t* __restrict__ h_st,
+                               int32_t* __restrict__ h_err) {
+  const int64_t words = cap / 16;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_items * words;
+       i += (int64_t)gridDim.x * blockDim.x)
+    reinterpret_cast<uint4*>(h_st)[i] =
+        reinterpret_cast<const uint4*>(items[i / words].st)[i % words];
+  if (blockIdx.x == 0 && threadIdx.x == 0) *h_err = *err;
+}
+
+// Counts and flags of a finished request into pinned host memory, and the
+// voltages of its first converged scenario into the feeder's warm start (one
+// block).
+__global__ void k_serve_done(const int32_t* __restrict__ iters, const uint8_t* __restrict__ conv,
+                             int B, const double2* __restrict__ V, int n,
+                             double2* __restrict__ warm, int32_t* __restrict__ h_it,
+                             uint8_t* __restrict__ h_cv) {
+  __shared__ int first;
+  if (threadIdx.x == 0) first = B;
+  __syncthreads();
+  int mine = B;
+  for (int b = threadIdx.x; b < B; b += blockDim.x) {
+    const uint8_t c = conv[b];
+    h_it[b] = iters[b];
+    h_cv[b] = c;
+    if (c && mine == B) mine = b;
+  }
+  if (mine < B) atomicMin(&first, mine);
+  __syncthreads();
+  if (first < B)
+    for (int j = threadIdx.x; j < n; j += blockDim.x) warm[j] = V[(int64_t)first * n + j];
+}
+
 struct Inflight {
   zbus_request req;
   int64_t s0;
@@ -78,7 +115,9 @@ struct Feeder {
   double2* res_V = nullptr;       // library result buffers [cap][n], [cap], [cap]
   int32_t* res_it = nullptr;
   uint8_t* res_cv = nullptr;
-  uint8_t* h_st = nullptr;        // pinned mirror of the slot states
+  uint8_t* h_st = nullptr;        // pinned mirrors: slot states, finished requests'
+  int32_t* h_it = nullptr;        // counts and flags (at the request's slots)
+  uint8_t* h_cv = nullptr;
 };
 
 int64_t first_fit(const std::vector<char>& used, int64_t B) {
@@ -199,17 +238,14 @@ extern "C" zbus_status zbus_serve(const zbus_serve_config* cfg, zbus_network* po
     group_free(&g);
     return s;
   }
-  int32_t* h_err = nullptr;
+  // everything the loop allocates besides the group: one device and one
+  // pinned allocation
+  char* d_slab = nullptr;
+  char* h_slab = nullptr;
   auto cleanup = [&]() {
     cudaStreamSynchronize(st);
-    cudaFreeHost(h_err);
-    for (auto& f : fd) {
-      cudaFree(f.warm);
-      cudaFree(f.res_V);
-      cudaFree(f.res_it);
-      cudaFree(f.res_cv);
-      cudaFreeHost(f.h_st);
-    }
+    cudaFree(d_slab);
+    cudaFreeHost(h_slab);
     group_free(&g);
   };
 #define SV_CHECK(call)          \
@@ -229,18 +265,44 @@ extern "C" zbus_status zbus_serve(const zbus_serve_config* cfg, zbus_network* po
       return _s;                                                              \
     }                                                                         \
   } while (0)
-  for (size_t k = 0; k < nets.size(); ++k) {
-    Feeder& f = fd[k];
-    f.cap = caps[k];
-    f.used.assign((size_t)f.cap, 0);
-    const size_t n = (size_t)nets[k]->n;
-    SV_CUDA(cudaMalloc((void**)&f.warm, n * sizeof(double2)));
-    SV_CUDA(cudaMalloc((void**)&f.res_V, (size_t)f.cap * n * sizeof(double2)));
-    SV_CUDA(cudaMalloc((void**)&f.res_it, (size_t)f.cap * sizeof(int32_t)));
-    SV_CUDA(cudaMalloc((void**)&f.res_cv, (size_t)f.cap));
-    SV_CUDA(cudaMallocHost((void**)&f.h_st, (size_t)f.cap));
+  size_t d_bytes = 0;
+  for (size_t k = 0; k < nets.size(); ++k)
+    d_bytes += (size_t)(cap + 1) * nets[k]->n * sizeof(double2) + (size_t)cap * 5;
+  SV_CUDA(cudaMalloc((void**)&d_slab, d_bytes));
+  SV_CUDA(cudaMallocHost((void**)&h_slab, (size_t)cap * 6 * nets.size() + sizeof(int32_t)));
+  {
+    char* dp = d_slab;
+    for (size_t k = 0; k < nets.size(); ++k) {   // 16-byte items, then 4, then 1
+      const size_t n = (size_t)nets[k]->n;
+      fd[k].cap = caps[k];
+      fd[k].used.assign((size_t)cap, 0);
+      fd[k].warm = (double2*)dp;
+      fd[k].res_V = fd[k].warm + n;
+      dp += (size_t)(cap + 1) * n * sizeof(double2);
+    }
+    for (auto& f : fd) {
+      f.res_it = (int32_t*)dp;
+      dp += (size_t)cap * sizeof(int32_t);
+    }
+    for (auto& f : fd) {
+      f.res_cv = (uint8_t*)dp;
+      dp += (size_t)cap;
+    }
+    char* hp = h_slab;
+    for (auto& f : fd) {
+      f.h_st = (uint8_t*)hp;
+      hp += (size_t)cap;
+    }
+    for (auto& f : fd) {
+      f.h_it = (int32_t*)hp;
+      hp += (size_t)cap * sizeof(int32_t);
+    }
+    for (auto& f : fd) {
+      f.h_cv = (uint8_t*)hp;
+      hp += (size_t)cap;
+    }
   }
-  SV_CUDA(cudaMallocHost((void**)&h_err, sizeof(int32_t)));
+  int32_t* const h_err = (int32_t*)(h_slab + (size_t)cap * 6 * nets.size());
   *h_err = 0;
   SV_CHECK(group_reset(&g, st));
   SV_CHECK(group_start(&g, cfg->tol, cfg->max_iter, cfg->conv_rule, nullptr, 0, st));
@@ -251,8 +313,6 @@ extern "C" zbus_status zbus_serve(const zbus_serve_config* cfg, zbus_network* po
   bool ended = false;
   bool source_failed = false;
   int64_t live_total = 0;
-  std::vector<int32_t> h_it;
-  std::vector<uint8_t> h_cv;
   int64_t n_pass = 0;
   while (true) {
     ++n_pass;
@@ -349,12 +409,9 @@ extern "C" zbus_status zbus_serve(const zbus_serve_config* cfg, zbus_network* po
       NvtxRange sweep_range("zbus_serve sweep");
       SV_CHECK(group_sweep(&g, 0, false, st));
     }
-    for (size_t k = 0; k < nets.size(); ++k)
-      if (!fd[k].live.empty())
-        SV_CUDA(cudaMemcpyAsync(fd[k].h_st, g.h_items[k].st, (size_t)fd[k].cap,
-                                cudaMemcpyDeviceToHost, st));
-    SV_CUDA(cudaMemcpyAsync(h_err, group_error_word(&g), sizeof(int32_t), cudaMemcpyDeviceToHost,
-                            st));
+    k_serve_status<<<(unsigned)std::min<int64_t>(64, (n_pool * (cap / 16) + 255) / 256), 256, 0,
+                     st>>>(g.d_items, n_pool, cap, group_error_word(&g), fd[0].h_st, h_err);
+    SV_CUDA(cudaGetLastError());
     SV_CUDA(cudaStreamSynchronize(st));
     if (*h_err != 0) SV_CHECK(group_device_status(&g, st));   // a device wait gave up
     // completions
@@ -383,6 +440,9 @@ extern "C" zbus_status zbus_serve(const zbus_serve_config* cfg, zbus_network* po
         uint8_t* cvp = fl.req.V_out && fl.req.converged ? fl.req.converged : f.res_cv + fl.s0;
         SV_CHECK(group_collect(&g, (int)k, fl.s0, fl.req.B, V, itp, cvp, fl.req.S_wye,
                                fl.req.S_delta, mtol, nullptr, cfg->max_correction, st));
+        k_serve_done<<<1, 256, 0, st>>>(itp, cvp, (int)fl.req.B, (const double2*)V, (int)n, f.warm,
+                                        f.h_it + fl.s0, f.h_cv + fl.s0);
+        SV_CUDA(cudaGetLastError());
         done.push_back(Done{k, fl, V, itp, cvp});
         f.live.erase(f.live.begin() + q);
       }
@@ -393,10 +453,8 @@ extern "C" zbus_status zbus_serve(const zbus_serve_config* cfg, zbus_network* po
     for (auto& d : done) {
       Feeder& f = fd[d.k];
       const int64_t B = d.fl.req.B;
-      h_it.resize((size_t)B);
-      h_cv.resize((size_t)B);
-      SV_CUDA(cudaMemcpy(h_it.data(), d.it, (size_t)B * sizeof(int32_t), cudaMemcpyDeviceToHost));
-      SV_CUDA(cudaMemcpy(h_cv.data(), d.cv, (size_t)B, cudaMemcpyDeviceToHost));
+      const int32_t* h_it = f.h_it + d.fl.s0;
+      const uint8_t* h_cv = f.h_cv + d.fl.s0;
       zbus_request_result res;
       std::memset(&res, 0, sizeof(res));
       res.status = ZBUS_OK;
@@ -406,18 +464,11 @@ extern "C" zbus_status zbus_serve(const zbus_serve_config* cfg, zbus_network* po
       res.V = d.V;
       res.iters = d.it;
       res.converged = d.cv;
-      int first_conv = -1;
       for (int64_t b = 0; b < B; ++b) {
-        res.n_converged += h_cv[(size_t)b] ? 1 : 0;
-        res.max_iters = std::max(res.max_iters, h_it[(size_t)b]);
-        if (first_conv < 0 && h_cv[(size_t)b]) first_conv = (int)b;
+        res.n_converged += h_cv[b] ? 1 : 0;
+        res.max_iters = std::max(res.max_iters, h_it[b]);
       }
-      if (first_conv >= 0) {
-        const size_t n = (size_t)nets[d.k]->n;
-        SV_CUDA(cudaMemcpy(f.warm, d.V + (size_t)first_conv * n * 2, n * sizeof(double2),
-                           cudaMemcpyDeviceToDevice));
-        f.warm_valid = true;
-      }
+      if (res.n_converged > 0) f.warm_valid = true;
       sink(user, &d.fl.req, &res);
       std::fill(f.used.begin() + d.fl.s0, f.used.begin() + d.fl.s0 + B, 0);
       live_total -= 1;
