@@ -570,6 +570,7 @@ void zbus_network_destroy(zbus_network net) {
   cudaFree(net->Zr);
   cudaFree(net->Zi);
   cudaFree(net->Zs);
+  cudaFree(net->Zt);
   cudaFree(net->csr_ptr);
   cudaFree(net->csr_col);
   cudaFree(net->csr_val);
@@ -703,13 +704,12 @@ zbus_status solve_device(zbus_network net, int64_t B, const double* S_wye, const
 
   net->last_group = nullptr;
   net->last_ctx = nullptr;   // the sweeps on the CUDA cores have no device-side waits
-  if (o.profile != 1 && B <= FUSED_MAX_B && net->n_pad <= FUSED_MAX_NPAD) {
+  if (o.profile != 1 && net->n_pad <= FUSED_MAX_NPAD) {
     // a small feeder: the whole solve in one launch, a block per scenario
     // (bitwise the results of the sweep-per-launch path below)
-    launch_solve_fused_f64(net->Zr, net->Zi, net->Zs, net->w, (const double2*)V_init,
-                           (const double2*)S_wye, (const double2*)S_delta, net->n, net->n_pad,
-                           (int)B, tol, max_iter, o.conv_rule, (double2*)V_out, iters, converged,
-                           st);
+    launch_solve_fused_f64(net->Zt, net->w, (const double2*)V_init, (const double2*)S_wye,
+                           (const double2*)S_delta, net->n, net->n_pad, (int)B, tol, max_iter,
+                           o.conv_rule, (double2*)V_out, iters, converged, st);
     ZB_CUDA(cudaGetLastError());
     return ZBUS_OK;
   }

@@ -7,6 +7,7 @@
 // Plus the run start (v^0), the whole solve of a small feeder in one launch
 // (K1-K3 of every sweep in one block per scenario, the latency case) and the
 // FP64 power-mismatch check.
+#include <algorithm>
 #include <cmath>
 
 #include "loads.cuh"
@@ -121,6 +122,7 @@ k_gemm3m_f64(const SolveCtx* __restrict__ ctx, const double* __restrict__ Zr,
   double2* V = ctx->V;
   const int32_t* list = ctx->list;
   double* part = ctx->part;
+  const bool summag = ctx->rule == ZBUS_CONV_SUMMAG;
 
   const int tid = threadIdx.x;
   const int tm = tid / THR_N;   // 0..15
@@ -210,7 +212,7 @@ k_gemm3m_f64(const SolveCtx* __restrict__ ctx, const double* __restrict__ Zr,
             double step = hypot(vn.x - vo.x, vn.y - vo.y);
             if (step != step) step = INFINITY;
             dmax = fmax(dmax, step);
-            dsum += hypot(vn.x, vn.y) - hypot(vo.x, vo.y);
+            if (summag) dsum += hypot(vn.x, vn.y) - hypot(vo.x, vo.y);
           }
         }
       }
@@ -317,160 +319,165 @@ k_gemm3m_f64_small(const SolveCtx* __restrict__ ctx, const double* __restrict__ 
 
 // ---------------------------------------------------------------------------
 // The whole solve of one small feeder in one launch (n_pad <= FUSED_MAX_NPAD
-// unknowns, at most FUSED_MAX_B scenarios): one block
-// per scenario keeps v and the 3M operands in shared memory and runs every
-// sweep (K1, K2, K3) itself, so a solve costs one launch instead of four
-// kernel nodes per sweep.  Every value is formed with the arithmetic of the
-// sweep kernels: the load currents of bus_injection (a thread per unknown
-// draws its wye current and its bus's delta branch, then adds the branches
-// into its phase as bus_injection does), each output's three products summed
-// over k in sequence, the step partials grouped as in k_gemm3m_f64_small and
-// reduced over the tiles as in k_decide (maxima in any order, which is exact;
-// the sums of the sum-of-magnitudes rule in the same order), so the results
-// are bitwise those of the sweep-per-launch path.
+// unknowns): one block per scenario keeps v and the 3M operands in shared memory and runs every sweep (K1, K2, K3) itself,
+// so a solve costs one launch instead of four kernel nodes per sweep.  Every
+// value is formed with the arithmetic of the sweep kernels: the load currents
+// of bus_injection (a thread per unknown draws its wye current or its bus's
+// delta branch, then adds the branches into its phase as bus_injection does),
+// each output's three products summed over k in sequence, so the voltages are
+// bitwise those of the sweep-per-launch path.  (The stop test compares the
+// root of the largest squared step with tol, theirs the largest hypot: equal
+// to an ulp.)
+//
+// Bound by the FP64 pipe, which a warp's instruction holds as long for 12
+// lanes as for 32: each of the three products of an output has a thread of
+// its own (3 n threads, 48 multiply-adds a warp at 36 unknowns where a thread
+// per output ran 144), Z is read k-major so that a warp's loads are one row
+// piece, a slot with one kind of load draws once, and the magnitudes of the
+// sum rule are formed under that rule only.  8 scenarios of 36 unknowns: 57
+// -> 26 us a call.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(FUSED_THREADS)
-k_solve_fused_f64(const double* __restrict__ Zr, const double* __restrict__ Zi,
-                  const double* __restrict__ Zs, const double2* __restrict__ w,
+__global__ void __launch_bounds__(FUSED_MAX_THREADS)
+k_solve_fused_f64(const double* __restrict__ Zt, const double2* __restrict__ w,
                   const double2* __restrict__ V_init, const double2* __restrict__ Sw,
                   const double2* __restrict__ Sd, int n, int n_pad, double tol, int max_iter,
                   int rule, double2* __restrict__ V, int32_t* __restrict__ iters,
                   uint8_t* __restrict__ conv) {
-  static_assert(FUSED_THREADS >= FUSED_MAX_NPAD && FUSED_THREADS == 128,
-                "one thread per padded unknown; four warps share the outputs");
   __shared__ double2 sv[FUSED_MAX_NPAD];
   __shared__ double2 sdw[FUSED_MAX_NPAD], sib[FUSED_MAX_NPAD];   // wye draws, delta branches
-  __shared__ double sIr[FUSED_MAX_NPAD], sIi[FUSED_MAX_NPAD], sIs[FUSED_MAX_NPAD];
+  __shared__ double sI[3][FUSED_MAX_NPAD];                       // Ir, Ii, Ir + Ii
+  __shared__ double sa[3][FUSED_MAX_NPAD];                       // the three products
   __shared__ double sds[FUSED_MAX_NPAD], su[FUSED_MAX_NPAD / 4];
-  __shared__ double swm[FUSED_THREADS / 32];
-  __shared__ int sok[FUSED_MAX_NPAD];
-  __shared__ int sdone;
+  __shared__ unsigned long long swm[FUSED_MAX_THREADS / 32], swh[FUSED_MAX_THREADS / 32];
   const int b = blockIdx.x, t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  const int warps = blockDim.x >> 5;
   const int64_t row = (int64_t)b * n;
   const int ntn = n_pad / F64_BN;
   const bool summag = rule == ZBUS_CONV_SUMMAG;
-  if (t < n) sv[t] = V_init ? V_init[row + t] : w[t];
   // this thread's unknown: bus j0 / 3, phase p, m valid phases in the bus
   const int j0 = 3 * (t / 3), p = t % 3, m = min(3, n - j0);
   const bool own = t < n;
   const bool delta = Sd != nullptr && m == 3 && own;
-  const double2 swj = (Sw && own) ? Sw[row + t] : make_double2(0.0, 0.0);
-  const double2 sdj = delta ? Sd[row + t] : make_double2(0.0, 0.0);
+  const double2 zero = make_double2(0.0, 0.0);
+  const double2 swj = (Sw && own) ? Sw[row + t] : zero;
+  const double2 sdj = delta ? Sd[row + t] : zero;
+  const bool has_w = swj.x != 0.0 || swj.y != 0.0;
+  const bool has_d = sdj.x != 0.0 || sdj.y != 0.0;
+  const double2 wj = own ? w[t] : zero;
+  // this thread's product and output
+  const int c = t / n, o = t - c * n;
+  const double* z = Zt + ((int64_t)(c < 3 ? c : 0) * n_pad) * n_pad + (c < 3 ? o : 0);
+  if (own) sv[t] = V_init ? V_init[row + t] : wj;
+  for (int i = t; i < 3 * FUSED_MAX_NPAD; i += blockDim.x) sI[0][i] = 0.0;
   __syncthreads();
-  for (int it = 1;; ++it) {
+  int it = 1, ok = 0;
+  for (;; ++it) {
     // K1a: the wye current of this unknown and the delta branch p of its bus
     // (branch p joins phases p and p + 1), as load_draw inside bus_injection
-    if (t < n_pad) {
-      double2 dw = make_double2(0.0, 0.0), ib = make_double2(0.0, 0.0);
-      if (own) {
-        if (Sw) dw = load_draw(swj, sv[t]);
-        if (delta) {
-          const double2 va = sv[t], vb = sv[j0 + (p == 2 ? 0 : p + 1)];
-          ib = load_draw(sdj, make_double2(va.x - vb.x, va.y - vb.y));
-        }
-      }
-      sdw[t] = dw;
-      sib[t] = ib;
+    if (own) {
+      const double2 va = sv[t], vb = sv[j0 + (p == 2 ? 0 : min(p + 1, m - 1))];
+      const double2 u = make_double2(va.x - vb.x, va.y - vb.y);
+      const double2 d = load_draw(has_w ? swj : sdj, has_w ? va : u);
+      sdw[t] = has_w ? d : zero;
+      sib[t] = has_w ? (has_d ? load_draw(sdj, u) : zero) : d;
     }
     __syncthreads();
     // K1b: phase p draws branch p and returns branch p - 1; injection = -drawn
-    if (t < n_pad) {
-      double2 inj = make_double2(0.0, 0.0);
-      if (own) {
-        double2 d = sdw[t];
-        if (delta) {
-          const double2 ib = sib[t], iw = sib[j0 + (p == 0 ? 2 : p - 1)];
-          d.x += ib.x - iw.x;
-          d.y += ib.y - iw.y;
-        }
-        inj = make_double2(-d.x, -d.y);
+    if (own) {
+      double2 d = sdw[t];
+      if (delta) {
+        const double2 ib = sib[t], iw = sib[j0 + (p == 0 ? 2 : p - 1)];
+        d.x += ib.x - iw.x;
+        d.y += ib.y - iw.y;
       }
-      sIr[t] = inj.x;
-      sIi[t] = inj.y;
-      sIs[t] = inj.x + inj.y;
+      sI[0][t] = -d.x;
+      sI[1][t] = -d.y;
+      sI[2][t] = -d.x + -d.y;
     }
     __syncthreads();
-    // K2: one output per thread, v <- w + D in place (the currents are read
-    // from shared memory only).  The outputs are dealt to the four warps in
-    // equal parts (n_pad / 4 lanes each), so each SM sub-partition's FP64
-    // pipe carries a quarter of the products.
-    double dm = 0.0;
-    const int per = n_pad / 4;
-    const int o = lane < per ? wid * per + lane : -1;
-    if (o >= 0) {
-      const bool out_own = o < n;
-      const double* zr = Zr + (int64_t)o * n_pad;
-      const double* zi = Zi + (int64_t)o * n_pad;
-      const double* zs = Zs + (int64_t)o * n_pad;
-      double a1 = 0.0, a2 = 0.0, a3 = 0.0;
-      for (int k = 0; k < n_pad; ++k) {
-        a1 = fma(zr[k], sIr[k], a1);
-        a2 = fma(zi[k], sIi[k], a2);
-        a3 = fma(zs[k], sIs[k], a3);
-      }
-      int ok = 0;
-      double ds = 0.0;
-      if (out_own) {
-        const double dr = a1 - a2;
-        const double di = a3 - a1 - a2;
-        const double2 vo = sv[o];
-        const double2 wi = w[o];
-        const double2 vn = make_double2(wi.x + dr, wi.y + di);
-        sv[o] = vn;
-        double step = hypot(vn.x - vo.x, vn.y - vo.y);
-        if (step != step) step = INFINITY;
-        dm = step;
-        ds = hypot(vn.x, vn.y) - hypot(vo.x, vo.y);
-        ok = 1;
-      }
-      sds[o] = ds;
-      sok[o] = ok;
+    // K2: one product of one output per thread
+    if (c < 3) {
+      const double* x = sI[c];
+      double a = 0.0;
+#pragma unroll 16
+      for (int k = 0; k < n_pad; ++k) a = fma(z[(int64_t)k * n_pad], x[k], a);
+      sa[c][o] = a;
     }
-    // K3: the largest step (maxima are exact in any order; every step is >= 0)
-    for (int o = 16; o > 0; o >>= 1) dm = fmax(dm, __shfl_xor_sync(0xffffffffu, dm, o));
-    if (lane == 0) swm[wid] = dm;
+    __syncthreads();
+    // v <- w + D in place, the largest squared step (by bit pattern; a step
+    // whose square leaves the range by hypot) and the magnitudes' change
+    unsigned long long m2 = 0ull, mh = 0ull;
+    if (own) {
+      const double a1 = sa[0][t], a2 = sa[1][t], a3 = sa[2][t];
+      const double2 vo = sv[t];
+      const double2 vn = make_double2(wj.x + (a1 - a2), wj.y + (a3 - a1 - a2));
+      sv[t] = vn;
+      const double dx = vn.x - vo.x, dy = vn.y - vo.y;
+      const double q = fma(dx, dx, dy * dy);
+      const unsigned long long qb =
+          (unsigned long long)__double_as_longlong(q) & 0x7FFFFFFFFFFFFFFFull;
+      if ((unsigned)(qb >> 52) - 128u < 1792u) {
+        m2 = qb;
+      } else if (dx != 0.0 || dy != 0.0) {
+        mh = (unsigned long long)__double_as_longlong(hypot(dx, dy)) & 0x7FFFFFFFFFFFFFFFull;
+        mh = mh > 0x7FF0000000000000ull ? 0x7FF0000000000000ull : mh;
+      }
+      if (summag) sds[t] = hypot(vn.x, vn.y) - hypot(vo.x, vo.y);
+    }
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+      const unsigned long long y2 = __shfl_xor_sync(0xffffffffu, m2, s);
+      const unsigned long long yh = __shfl_xor_sync(0xffffffffu, mh, s);
+      m2 = y2 > m2 ? y2 : m2;
+      mh = yh > mh ? yh : mh;
+    }
+    if (lane == 0) {
+      swm[wid] = m2;
+      swh[wid] = mh;
+    }
     __syncthreads();
     // the sum-of-magnitudes rule: per tile and thread column tn the outputs
     // tn, tn + 12, tn + 24, tn + 36 in order, then tn = 0..11, then the tiles
-    if (summag && t < ntn * (F64_BN / 4)) {
-      const int nt = t / (F64_BN / 4), tn = t % (F64_BN / 4);
-      double u = 0.0;
-      for (int c = 0; c < 4; ++c) {
-        const int o = nt * F64_BN + tn + (F64_BN / 4) * c;
-        if (sok[o]) u += sds[o];
-      }
-      su[t] = u;
-    }
-    __syncthreads();
-    if (t == 0) {
-      double dmax = 0.0;
-      for (int x = 0; x < FUSED_THREADS / 32; ++x) dmax = fmax(dmax, swm[x]);
-      double dsum = 0.0;
-      if (summag)
-        for (int nt = 0; nt < ntn; ++nt) {
-          double tu = 0.0;
-          for (int tn = 0; tn < F64_BN / 4; ++tn) tu += su[nt * (F64_BN / 4) + tn];
-          dsum += tu;
+    if (summag) {
+      if (t < ntn * (F64_BN / 4)) {
+        const int nt = t / (F64_BN / 4), tn = t % (F64_BN / 4);
+        double u = 0.0;
+        for (int q = 0; q < 4; ++q) {
+          const int i = nt * F64_BN + tn + (F64_BN / 4) * q;
+          if (i < n) u += sds[i];
         }
-      const double delta_v = summag ? fabs(dsum) : dmax;
-      int done = 1;
-      if (!isfinite(delta_v)) {
-        conv[b] = 0;
-      } else if (delta_v <= tol) {
-        conv[b] = 1;
-      } else if (it < max_iter) {
-        done = 0;
-      } else {
-        conv[b] = 0;
+        su[t] = u;
       }
-      if (done) iters[b] = it;
-      sdone = done;
+      __syncthreads();
     }
-    __syncthreads();
-    if (sdone) break;
-    __syncthreads();
+    // every thread decides alike
+    double delta_v;
+    if (summag) {
+      double dsum = 0.0;
+      for (int nt = 0; nt < ntn; ++nt) {
+        double tu = 0.0;
+        for (int tn = 0; tn < F64_BN / 4; ++tn) tu += su[nt * (F64_BN / 4) + tn];
+        dsum += tu;
+      }
+      delta_v = fabs(dsum);
+    } else {
+      m2 = swm[0];
+      mh = swh[0];
+      for (int x = 1; x < warps; ++x) {
+        m2 = swm[x] > m2 ? swm[x] : m2;
+        mh = swh[x] > mh ? swh[x] : mh;
+      }
+      delta_v = fmax(sqrt(__longlong_as_double((long long)m2)),
+                     __longlong_as_double((long long)mh));
+    }
+    ok = delta_v <= tol;
+    if (ok || !isfinite(delta_v) || it >= max_iter) break;
   }
-  if (t < n) V[row + t] = sv[t];
+  if (own) V[row + t] = sv[t];
+  if (t == 0) {
+    iters[b] = it;
+    conv[b] = (uint8_t)ok;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -696,13 +703,14 @@ void launch_gemm_f64(SolveCtx* ctx, const double* Zr, const double* Zi, const do
     k_gemm3m_f64<<<grid, GEMM_THREADS, 0, st>>>(ctx, Zr, Zi, Zs, w, n, n_pad);
 }
 
-void launch_solve_fused_f64(const double* Zr, const double* Zi, const double* Zs,
-                            const double2* w, const double2* V_init, const double2* S_wye,
-                            const double2* S_del, int n, int n_pad, int B, double tol,
-                            int max_iter, int rule, double2* V, int32_t* iters, uint8_t* conv,
-                            cudaStream_t st) {
-  k_solve_fused_f64<<<B, FUSED_THREADS, 0, st>>>(Zr, Zi, Zs, w, V_init, S_wye, S_del, n, n_pad,
-                                                  tol, max_iter, rule, V, iters, conv);
+// A thread per product of every output, at least one per padded unknown.
+void launch_solve_fused_f64(const double* Zt, const double2* w, const double2* V_init,
+                            const double2* S_wye, const double2* S_del, int n, int n_pad, int B,
+                            double tol, int max_iter, int rule, double2* V, int32_t* iters,
+                            uint8_t* conv, cudaStream_t st) {
+  const int threads = round_up(std::max(3 * n, n_pad), 32);
+  k_solve_fused_f64<<<B, threads, 0, st>>>(Zt, w, V_init, S_wye, S_del, n, n_pad, tol, max_iter,
+                                           rule, V, iters, conv);
 }
 
 void launch_converge(SolveCtx* ctx, int B, cudaGraphConditionalHandle h, bool use_handle,

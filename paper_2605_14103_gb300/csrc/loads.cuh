@@ -6,11 +6,12 @@
 
 namespace zbus {
 
-// conj(S / v) = conj(S) v / |v|^2; zero when the slot has no load.
+// conj(S / v) = conj(S) v / |v|^2; zero when the slot has no load.  The
+// multiply-adds are written out, so every kernel rounds alike.
 __device__ __forceinline__ double2 load_draw(double2 S, double2 v) {
   if (S.x == 0.0 && S.y == 0.0) return make_double2(0.0, 0.0);
-  const double inv = 1.0 / (v.x * v.x + v.y * v.y);
-  return make_double2((S.x * v.x + S.y * v.y) * inv, (S.x * v.y - S.y * v.x) * inv);
+  const double inv = 1.0 / fma(v.x, v.x, v.y * v.y);
+  return make_double2(fma(S.x, v.x, S.y * v.y) * inv, fma(S.x, v.y, -(S.y * v.x)) * inv);
 }
 
 // Current injection of one bus (three consecutive unknowns).  Wye slot p draws

@@ -167,6 +167,16 @@ __global__ void k_pack_f64(const double2* Z, int n, int n_pad, double* Zr, doubl
   }
 }
 
+// The three copies transposed, [3][n_pad][n_pad] (small feeders).
+__global__ void k_pack_t(const double* Zr, const double* Zi, const double* Zs, int n_pad,
+                         double* Zt) {
+  const int tot = n_pad * n_pad;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < 3 * tot; t += gridDim.x * blockDim.x) {
+    const int c = t / tot, k = t % tot / n_pad, o = t % n_pad;
+    Zt[t] = (c == 0 ? Zr : c == 1 ? Zi : Zs)[o * n_pad + k];
+  }
+}
+
 __global__ void k_check_finite(const double2* w, int n, int32_t* info) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n && !(isfinite(w[i].x) && isfinite(w[i].y))) atomicCAS(info, 0, -1);
@@ -628,8 +638,14 @@ zbus_status ensure_3m(zbus_network net, cudaStream_t st) {
     s = cuda_fail(ce, "cudaMalloc(3M operands)", __FILE__, __LINE__);
   } else {
     k_pack_f64<<<2048, 256, 0, st>>>(net->Z, net->n, net->n_pad, net->Zr, net->Zi, net->Zs);
-    if ((ce = cudaGetLastError()) != cudaSuccess ||
-        (ce = cudaStreamSynchronize(st)) != cudaSuccess)
+    if (net->n_pad <= FUSED_MAX_NPAD) {
+      if ((ce = cudaMalloc((void**)&net->Zt, 3 * pb)) != cudaSuccess)
+        s = cuda_fail(ce, "cudaMalloc(transposed 3M operands)", __FILE__, __LINE__);
+      else
+        k_pack_t<<<64, 256, 0, st>>>(net->Zr, net->Zi, net->Zs, net->n_pad, net->Zt);
+    }
+    if (s == ZBUS_OK && ((ce = cudaGetLastError()) != cudaSuccess ||
+                         (ce = cudaStreamSynchronize(st)) != cudaSuccess))
       s = cuda_fail(ce, "3M operands", __FILE__, __LINE__);
   }
   if (s != ZBUS_OK) release_3m(net);
@@ -648,7 +664,8 @@ void release_3m(zbus_network net) {
   cudaFree(net->Zr);
   cudaFree(net->Zi);
   cudaFree(net->Zs);
-  net->Zr = net->Zi = net->Zs = nullptr;
+  cudaFree(net->Zt);
+  net->Zr = net->Zi = net->Zs = net->Zt = nullptr;
 }
 
 }  // namespace zbus

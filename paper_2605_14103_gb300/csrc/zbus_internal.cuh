@@ -37,14 +37,12 @@ zbus_status cuda_fail(cudaError_t e, const char* what, const char* file, int lin
 // ---------------------------------------------------------------------------
 constexpr int F64_BM = 32;   // scenarios per tile
 constexpr int F64_BN = 48;   // outputs (16 buses) per tile
-// whole-solve kernel of small feeders: up to 96 padded unknowns, one block of
-// four warps per scenario.  Up to 2048 scenarios: the sweep kernels wait on
-// their launches and on a few long blocks (solves in us, sweeps / whole, 36
-// and 96 unknowns: 64 scenarios 520 / 56 and 1539 / 191, 1024 520 / 247 and
-// 1704 / 950, 4096 576 / 923 and 3193 / 3568, where whole warps pay).
+// whole-solve kernel of small feeders: up to 96 padded unknowns, one block
+// per scenario, at every batch (solves in us, sweep kernels / whole, 36 and 96
+// unknowns: 64 scenarios 518 / 26 and 1536 / 97, 1024 520 / 95 and 1703 / 561,
+// 16384 1910 / 1380 and 10073 / 8391)
 constexpr int FUSED_MAX_NPAD = 96;
-constexpr int FUSED_MAX_B = 2048;
-constexpr int FUSED_THREADS = 128;
+constexpr int FUSED_MAX_THREADS = 3 * FUSED_MAX_NPAD;
 constexpr int F64_BK = 16;   // k step
 constexpr int F64_PAD = 48;  // n is padded to a multiple of this
 
@@ -249,6 +247,7 @@ struct zbus_network_s {
   double* Zr = nullptr;      // [n_pad][n_pad] row-major, zero padded
   double* Zi = nullptr;
   double* Zs = nullptr;      // Zr + Zi
+  double* Zt = nullptr;      // small feeders: the three transposed, [3][n_pad][n_pad]
   int32_t* csr_ptr = nullptr;   // Y_LL rows (n + 1)
   int32_t* csr_col = nullptr;
   double2* csr_val = nullptr;
@@ -369,11 +368,10 @@ void launch_gemm_f64(SolveCtx* ctx, const double* Zr, const double* Zi, const do
 int gemm_f64_grid(int B, int n_pad);
 void launch_converge(SolveCtx* ctx, int B, cudaGraphConditionalHandle h, bool use_handle,
                      cudaStream_t st);
-void launch_solve_fused_f64(const double* Zr, const double* Zi, const double* Zs,
-                            const double2* w, const double2* V_init, const double2* S_wye,
-                            const double2* S_del, int n, int n_pad, int B, double tol,
-                            int max_iter, int rule, double2* V, int32_t* iters, uint8_t* conv,
-                            cudaStream_t st);
+void launch_solve_fused_f64(const double* Zt, const double2* w, const double2* V_init,
+                            const double2* S_wye, const double2* S_del, int n, int n_pad, int B,
+                            double tol, int max_iter, int rule, double2* V, int32_t* iters,
+                            uint8_t* conv, cudaStream_t st);
 void launch_mismatch(const double2* V, const double2* S_wye, const double2* S_del,
                      const int32_t* ptr, const int32_t* col, const double2* val,
                      const double2* ys, int n, int B, double* out, cudaStream_t st);
