@@ -17,7 +17,7 @@
 //
 // Measured per sweep against the FP64 contraction (k_currents_f64 +
 // k_gemm3m_f64 + the stop test): 1000 scenarios of 3069 unknowns 66 -> 1.35 ms
-// (contraction 1.03), 4096 of 381 3.5 -> 0.29 ms (0.085).  Error of one map
+// (contraction 1.03), 4096 of 381 3.5 -> 0.24 ms (0.085).  Error of one map
 // against extended precision, 102 to 2397 unknowns: 0.99 to 0.43 of the FP64
 // contraction's root mean square; of one adjoint sweep 0.70 to 0.28.
 //
@@ -325,47 +325,45 @@ __device__ __forceinline__ long long fixed_point(double x, int e) {
 
 // Slices of one row of n complex values, by all threads of the block: digit p
 // of component c of value(j) goes to plane c * 7 + p of out, `plane` halves
-// apart, eight columns at a time.
+// apart; a thread takes four columns of one component at a time.
 template <typename Load>
 __device__ __forceinline__ void write_slices(Load value, int n, int K_pad, int e, __half* out,
                                              int64_t plane) {
   const __half2 bias = __floats2half2_rn(1280.f, 1280.f);
-  for (int g = threadIdx.x; g < K_pad / 8; g += blockDim.x) {
-#pragma unroll 1
-    for (int c = 0; c < 3; ++c) {
-      long long y[8];
+  const int groups = K_pad / 4;
+  for (int u = threadIdx.x; u < 3 * groups; u += blockDim.x) {
+    const int c = u / groups, g = u - c * groups;
+    long long y[4];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int j = g * 8 + i;
-        const double2 v = j < n ? value(j) : make_double2(0.0, 0.0);
-        y[i] = 0;
-        if (c != 1) y[i] += fixed_point(v.x, e);
-        if (c != 0) y[i] += fixed_point(v.y, e);
-      }
-      __half* dst = out + (int64_t)c * SPLIT_S * plane + g * 8;
+    for (int i = 0; i < 4; ++i) {
+      const int j = g * 4 + i;
+      const double2 v = j < n ? value(j) : make_double2(0.0, 0.0);
+      y[i] = fixed_point(c == 1 ? v.y : v.x, e);
+      if (c == 2) y[i] += fixed_point(v.y, e);
+    }
+    __half* dst = out + (int64_t)c * SPLIT_S * plane + g * 4;
 #pragma unroll
-      for (int p = SPLIT_S - 1; p >= 0; --p) {
-        uint32_t w[4];
+    for (int p = SPLIT_S - 1; p >= 0; --p) {
+      uint32_t w[2];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          uint32_t pair = 0x64006400u;   // the halves 1024 + (digit + 256), minus 1280 below
+      for (int i = 0; i < 2; ++i) {
+        uint32_t pair = 0x64006400u;   // the halves 1024 + (digit + 256), minus 1280 below
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            long long& v = y[2 * i + h];
-            int d;
-            if (p > 0) {
-              d = (int)(((uint32_t)v + 128u) & 255u) - 128;
-              v = (v - d) >> 8;
-            } else {
-              d = (int)v;   // at most 256 in magnitude
-            }
-            pair += (uint32_t)(d + 256) << (16 * h);
+        for (int h = 0; h < 2; ++h) {
+          long long& v = y[2 * i + h];
+          int d;
+          if (p > 0) {
+            d = (int)(((uint32_t)v + 128u) & 255u) - 128;
+            v = (v - d) >> 8;
+          } else {
+            d = (int)v;   // at most 256 in magnitude
           }
-          const __half2 hv = __hsub2(*reinterpret_cast<const __half2*>(&pair), bias);
-          w[i] = *reinterpret_cast<const uint32_t*>(&hv);
+          pair += (uint32_t)(d + 256) << (16 * h);
         }
-        *reinterpret_cast<uint4*>(dst + p * plane) = make_uint4(w[0], w[1], w[2], w[3]);
+        const __half2 hv = __hsub2(*reinterpret_cast<const __half2*>(&pair), bias);
+        w[i] = *reinterpret_cast<const uint32_t*>(&hv);
       }
+      *reinterpret_cast<uint2*>(dst + p * plane) = make_uint2(w[0], w[1]);
     }
   }
 }
@@ -412,10 +410,16 @@ k_split_pack(const double* __restrict__ Zr, const double* __restrict__ Zi, int n
 // Update, stop test and next operand, one block per active scenario.
 //   v_i <- w_i + 2^(ez_i + ex_b - 62) sum_d D_d 2^(8 (6 - d))
 // with the three components combined as integers (T1 - T2, T3 - T1 - T2) in
-// two 64-bit words of four and three digit weights, exact until one rounding.  The block then holds the scenario's new voltages, so it
-// decides the stop and, if the scenario goes on, takes a slot of the next
-// sweep and writes the slices of i(v) (or of conj(lambda)) there.  The slot
-// order may differ between runs; no result depends on it.
+// two 64-bit words of four and three digit weights, exact until one rounding.
+// The block then holds the scenario's new voltages, so it decides the stop
+// and, if the scenario goes on, takes a slot of the next sweep and writes the
+// slices of i(v) (or of conj(lambda)) there.  The slot order may differ
+// between runs; no result depends on it.
+//
+// Bound by the FP64 pipe (about 34 operations an unknown at two a clock and
+// SM: 91 us for 4096 scenarios of 381 unknowns) and by the latencies between
+// the block's barriers: 156 us there, 203 before the voltages had a thread per
+// unknown and the slices one per four columns.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double exact_double(long long x) {   // |x| < 2^51
   return __longlong_as_double(x + 0x4338000000000000ll) - 6755399441055744.0;
@@ -454,8 +458,13 @@ __device__ __forceinline__ void operand_of_bus(const SolveCtx& c, int b, int n, 
     if (p >= m) x[p] = make_double2(0.0, 0.0);
 }
 
+// Blocks of 256 threads an SM holds: at 2 the FP64 pipe waits (176 us a sweep
+// of 4096 scenarios of 381 unknowns against 156), at 4 the spills cost a few
+// scenarios (92 us a sweep of 16 of 3069 unknowns against 76).
+constexpr int STEP_MIN = 3;
+
 template <bool ADJ, bool FIRST>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, STEP_MIN)
 k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs,
              const double2* __restrict__ w, int n, int K_pad, int64_t rows,
              cudaGraphConditionalHandle h, int use_handle) {
@@ -463,7 +472,7 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs,
   __shared__ unsigned long long red[8];
   __shared__ double sred[8];
   __shared__ int s_keep, s_slot;
-  const SolveCtx c = *ctx;
+  const SolveCtx& c = *ctx;
   const int tid = threadIdx.x;
   const int ld = (n + 7) & ~7;
   const int nb = (n + 2) / 3;
@@ -474,7 +483,8 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs,
   double* const xs_out = c.xs + (int64_t)(FIRST ? par : par ^ 1) * rows;
   const int it = c.iter + 1;
   const bool summag = c.rule == ZBUS_CONV_SUMMAG;
-  for (int slot = blockIdx.x; slot < c.count; slot += gridDim.x) {
+  const int count = c.count;
+  for (int slot = blockIdx.x; slot < count; slot += gridDim.x) {
     const int b = list[slot];
     const bool in = ZB_IN(b, c.B, 0x501u);
     int out_slot = slot;
@@ -485,57 +495,44 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs,
     double dsum = 0.0;
     const double xb = FIRST ? 0.0 : xs[slot];
     const double inv_s = ADJ ? 1.0 / c.gscale[in ? b : 0] : 0.0;
+    // voltages, a thread per unknown
     if (in)
-      for (int k = tid; k < nb; k += blockDim.x) {
-        const int j0 = 3 * k, m = min(3, n - j0);
-        double2 v[3];
-#pragma unroll
-        for (int p = 0; p < 3; ++p) {
-          const int j = j0 + p;
-          v[p] = make_double2(1.0, 0.0);
-          if (p >= m) continue;
-          const double2 vo = V[j];
-          if (FIRST) {
-            v[p] = vo;
-            continue;
-          }
-          const int32_t* D = c.D + (int64_t)slot * ld + j;
-          const int64_t plane = rows * ld;
-          long long hi[3], lo[3];
-#pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            int32_t t[SPLIT_S];
-#pragma unroll
-            for (int d = 0; d < SPLIT_S; ++d) t[d] = D[(q * SPLIT_S + d) * plane];
-            hi[q] = ((long long)t[0] << 24) + ((long long)t[1] << 16) + ((long long)t[2] << 8) +
-                    t[3];
-            lo[q] = ((long long)t[4] << 16) + ((long long)t[5] << 8) + t[6];
-          }
-          const double re = recombine(hi[0] - hi[1], lo[0] - lo[1]);
-          const double im = recombine(hi[2] - hi[0] - hi[1], lo[2] - lo[0] - lo[1]);
-          const double s = zs[j] * xb;
-          const double2 wj = ADJ ? make_double2(0.0, 0.0) : w[j];
-          v[p] = make_double2(fma(re, s, wj.x), fma(im, s, wj.y));
-          V[j] = v[p];
-          const double dx = v[p].x - vo.x, dy = v[p].y - vo.y;
-          const double q2 = fma(dx, dx, dy * dy);
-          const unsigned long long qb = abs_bits(q2);
-          if ((unsigned)(qb >> 52) - 128u < 1792u) {   // far inside the range of squares
-            st2 = max_u64(st2, qb);
-          } else if ((abs_bits(dx) | abs_bits(dy)) != 0ull) {
-            const unsigned long long hb = abs_bits(hypot(dx, dy));
-            sth = max_u64(sth, hb > 0x7FF0000000000000ull ? 0x7FF0000000000000ull : hb);
-          }
-          if (summag) dsum += hypot(v[p].x, v[p].y) - hypot(vo.x, vo.y);
+      for (int j = tid; j < n; j += blockDim.x) {
+        if (FIRST) {
+          op[j] = V[j];
+          continue;
         }
-        double2 x[3];
-        operand_of_bus<ADJ>(c, b, n, j0, m, inv_s, v, x);
+        const int32_t* D = c.D + (int64_t)slot * ld + j;
+        const int64_t plane = rows * ld;
+        int32_t t[3][SPLIT_S];
 #pragma unroll
-        for (int p = 0; p < 3; ++p)
-          if (p < m) {
-            op[j0 + p] = x[p];
-            top = max_u64(top, max_u64(abs_bits(x[p].x), abs_bits(x[p].y)));
-          }
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+          for (int d = 0; d < SPLIT_S; ++d) t[q][d] = D[(q * SPLIT_S + d) * plane];
+        const double2 vo = V[j];
+        const double2 wj = ADJ ? make_double2(0.0, 0.0) : w[j];
+        const double s = zs[j] * xb;
+        long long hi[3], lo[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          hi[q] = ((long long)t[q][0] << 24) + ((long long)t[q][1] << 16) +
+                  ((long long)t[q][2] << 8) + t[q][3];
+          lo[q] = ((long long)t[q][4] << 16) + ((long long)t[q][5] << 8) + t[q][6];
+        }
+        const double re = recombine(hi[0] - hi[1], lo[0] - lo[1]);
+        const double im = recombine(hi[2] - hi[0] - hi[1], lo[2] - lo[0] - lo[1]);
+        const double2 v = make_double2(fma(re, s, wj.x), fma(im, s, wj.y));
+        V[j] = v;
+        op[j] = v;
+        const double dx = v.x - vo.x, dy = v.y - vo.y;
+        const unsigned long long qb = abs_bits(fma(dx, dx, dy * dy));
+        if ((unsigned)(qb >> 52) - 128u < 1792u) {   // far inside the range of squares
+          st2 = max_u64(st2, qb);
+        } else if ((abs_bits(dx) | abs_bits(dy)) != 0ull) {
+          const unsigned long long hb = abs_bits(hypot(dx, dy));
+          sth = max_u64(sth, hb > 0x7FF0000000000000ull ? 0x7FF0000000000000ull : hb);
+        }
+        if (summag) dsum += hypot(v.x, v.y) - hypot(vo.x, vo.y);
       }
     if (!FIRST) {
       st2 = block_max_u64(st2, red);
@@ -578,7 +575,24 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs,
         continue;
       }
       out_slot = s_slot;
+    } else {
+      __syncthreads();
     }
+    // operand in their place, a thread per bus
+    if (in)
+      for (int k = tid; k < nb; k += blockDim.x) {
+        const int j0 = 3 * k, m = min(3, n - j0);
+        double2 v[3], x[3];
+#pragma unroll
+        for (int p = 0; p < 3; ++p) v[p] = p < m ? op[j0 + p] : make_double2(1.0, 0.0);
+        operand_of_bus<ADJ>(c, b, n, j0, m, inv_s, v, x);
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+          if (p < m) {
+            op[j0 + p] = x[p];
+            top = max_u64(top, max_u64(abs_bits(x[p].x), abs_bits(x[p].y)));
+          }
+      }
     top = block_max_u64(top, red);
     // a value that is not finite: the scale carries it to every output
     const bool bad = top >= 0x7FF0000000000000ull;
@@ -602,7 +616,7 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs,
     if (atomicAdd(&ctx->done, 1) == (int)gridDim.x - 1) {
       __threadfence();
       const int left = atomicAdd(&ctx->next, 0);
-      if (c.hist && c.iter < c.hist_n) c.hist[c.iter] = c.count;
+      if (c.hist && it - 1 < c.hist_n) c.hist[it - 1] = count;
       ctx->count = left;
       ctx->iter = it;
       ctx->next = 0;
