@@ -1646,9 +1646,11 @@ k_screen(const ItemDesc* __restrict__ items, int k, int s0, const float* __restr
   const int32_t* __restrict__ bcol = it.bsr_col;
   const float4* __restrict__ bval = it.bsr_df;
   unsigned long long worst = 0ull;
-  // runs of CHUNK_BUS buses per warp: neighbours in index often share a line
-  for (int a0 = (by * CHECK_WARPS + ty) * CHUNK_BUS; a0 < nb; a0 += ny * CHECK_WARPS * CHUNK_BUS)
-    for (int a = a0; a < min(nb, a0 + CHUNK_BUS); ++a) {
+  // runs of up to CHUNK_BUS buses per warp (neighbours in index often share a
+  // line), one bus each while the grid's warps outnumber the buses
+  const int run = max(1, min(CHUNK_BUS, nb / (ny * CHECK_WARPS)));
+  for (int a0 = (by * CHECK_WARPS + ty) * run; a0 < nb; a0 += ny * CHECK_WARPS * run)
+    for (int a = a0; a < min(nb, a0 + run); ++a) {
       float2 ah3[3], al3[3], sw[3], sd[3], acc[3];
       float va = 0.f;
 #pragma unroll
