@@ -162,6 +162,31 @@ __global__ void k_group_params(GroupState* gs, double tol, int max_iter, int rul
   gs->err = 0;
 }
 
+// Brings a bus's state and loads (32 slots) to L2, a lane a 128-byte line: 12
+// of the state, 6 of each kind of load.  Where the state does not stay in L2
+// (far), a warp asks for its next bus before it works on this one: the loads
+// at the top of a bus then wait for L2 and not for memory, and hold no
+// registers for it.  1024 buses x 16384: a FP32 residual 580 -> 520 us, in
+// double-float 935 -> 909; the neighbours' lines too: 541 / 945; a state that
+// L2 holds only pays for the instructions.
+struct BusAhead {
+  const char* line;
+  int stride;
+  __device__ BusAhead(const ItemDesc& it, int64_t base, int lane, bool far) {
+    const int l = lane < 12 ? lane : (lane - 12) % 6;
+    const int64_t first = base - lane;   // the warp's slot 0
+    const char* v = reinterpret_cast<const char*>(it.V4 + first + SLOT_BLOCK * (l >> 2));
+    const char* s = reinterpret_cast<const char*>((lane < 18 ? it.Swf : it.Sdf) + first +
+                                                  SLOT_BLOCK * (l >> 1));
+    line = lane < 12 ? v + 128 * (l & 3) : s + 128 * (l & 1);
+    stride = 3 * SLOT_BLOCK * (lane < 12 ? (int)sizeof(float4) : (int)sizeof(float2));
+    if (!far || lane >= 24) line = nullptr;
+  }
+  __device__ __forceinline__ void fetch(int a) const {
+    if (line) asm volatile("prefetch.global.L2 [%0];" :: "l"(line + (int64_t)a * stride));
+  }
+};
+
 // One block of the FP32 residual: J = Y_ab d (d = v_b - v_a, the slack's
 // voltage minus v_a, or v_a itself for the shunt term) with the hi part of
 // Y, added to acc, the largest |Re J|, |Im J| kept in mag.
@@ -239,9 +264,12 @@ k_residual_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
   const int rows_pad = OUT == RES_F32 ? it.n : it.K_pad >> 1;
   const int nchunks = (rows_pad + CHUNK_ROWS - 1) / CHUNK_ROWS;
   float amax = 0.f, mag = 0.f;
+  const BusAhead ahead(it, base, lane, gs->stream_state != 0);
   for (int ch = ys * RES_WARPS + warp; ch < nchunks; ch += split * RES_WARPS) {
     for (int q = 0; q < CHUNK_BUS; ++q) {
       const int a = ch * CHUNK_BUS + q;
+      const int an = q + 1 < CHUNK_BUS ? a + 1 : (ch + split * RES_WARPS) * CHUNK_BUS;
+      if (an < nb) ahead.fetch(an);
       float2 r[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
       if (a < nb && act) {
         float2 ah3[3], al3[3], sw[3], sd[3], inj[3], injl[3];   // own state, loads
@@ -1522,7 +1550,7 @@ k_check(const double2* __restrict__ V, const double2* __restrict__ Sw,
 // which is above mtol exactly when the largest of all is.
 //
 // Bound by the latency of the neighbours' state loads, like the FP32 start
-// sweeps: 0.8 ms for 16384 scenarios of 1023 buses against 3.6 for k_branch_f64
+// sweeps: 0.72 ms for 16384 scenarios of 1023 buses against 3.6 for k_branch_f64
 // + k_check, which the FP64 pipe bounds.
 // ---------------------------------------------------------------------------
 constexpr float U32 = 0x1p-24f;
@@ -1625,7 +1653,7 @@ __device__ __noinline__ unsigned long long screen_bus_f64(
 }
 
 __global__ void __launch_bounds__(32 * CHECK_WARPS, 6)
-k_screen(const ItemDesc* __restrict__ items, int k, int s0, const float* __restrict__ ynorm,
+k_screen(const GroupState* __restrict__ gs, const ItemDesc* __restrict__ items, int k, int s0, const float* __restrict__ ynorm,
          float mt2, const double2* __restrict__ V, const double2* __restrict__ Sw64,
          const double2* __restrict__ Sd64, const uint8_t* __restrict__ conv, int B,
          const double2* __restrict__ bval64, double2 vs0, double2 vs1, double2 vs2,
@@ -1649,8 +1677,11 @@ k_screen(const ItemDesc* __restrict__ items, int k, int s0, const float* __restr
   // runs of up to CHUNK_BUS buses per warp (neighbours in index often share a
   // line), one bus each while the grid's warps outnumber the buses
   const int run = max(1, min(CHUNK_BUS, nb / (ny * CHECK_WARPS)));
+  const BusAhead ahead(it, base, lane, gs->stream_state != 0);
   for (int a0 = (by * CHECK_WARPS + ty) * run; a0 < nb; a0 += ny * CHECK_WARPS * run)
     for (int a = a0; a < min(nb, a0 + run); ++a) {
+      const int an = a + 1 < a0 + run ? a + 1 : a0 + ny * CHECK_WARPS * run;
+      if (an < nb) ahead.fetch(an);
       float2 ah3[3], al3[3], sw[3], sd[3], acc[3];
       float va = 0.f;
 #pragma unroll
@@ -2507,7 +2538,7 @@ zbus_status group_collect(Group* g, int k, int64_t s0, int64_t B, double* V_out,
   if (!mm_out && mtol >= SCREEN_MIN_TOL && mtol <= 1e12) {
     const float mt2 = (float)(mtol * mtol) * 0.9999f;
     k_screen<<<(unsigned)((int64_t)gx * ny), dim3(32, CHECK_WARPS), 0, st>>>(
-        g->d_items, k, (int)s0, net->bsr_norm, mt2, (const double2*)V_out, (const double2*)S_wye,
+        g->d_state, g->d_items, k, (int)s0, net->bsr_norm, mt2, (const double2*)V_out, (const double2*)S_wye,
         (const double2*)S_delta, converged, (int)B, net->bsr_val, net->v_slack[0],
         net->v_slack[1], net->v_slack[2], mmax, ny);
   } else {
