@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include "loads.cuh"
+
 namespace zbus {
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
@@ -19,7 +21,7 @@ __device__ __forceinline__ double2 csub(double2 a, double2 b) {
 
 // conj(S / u^2) = conj(S) u^2 / |u|^4; zero for an absent load.
 __device__ __forceinline__ double2 load_slope(double2 S, double2 u) {
-  if (S.x == 0.0 && S.y == 0.0) return make_double2(0.0, 0.0);
+  if (!has_load(S)) return make_double2(0.0, 0.0);
   const double q = u.x * u.x + u.y * u.y;
   const double2 u2 = cmul(u, u);
   const double2 r = cmul(cconj(S), u2);
@@ -45,8 +47,8 @@ __device__ __forceinline__ void adjoint_rhs(const double2* v, const double2* mu,
   bool wye = false, delta = false;
 #pragma unroll
   for (int p = 0; p < 3; ++p) {
-    wye = wye || sw[p].x != 0.0 || sw[p].y != 0.0;
-    delta = delta || sd[p].x != 0.0 || sd[p].y != 0.0;
+    wye = wye || has_load(sw[p]);
+    delta = delta || has_load(sd[p]);
   }
   delta = delta && m == 3;
   double2 lam[3];

@@ -361,8 +361,8 @@ k_solve_fused_f64(const double* __restrict__ Zt, const double2* __restrict__ w,
   const double2 zero = make_double2(0.0, 0.0);
   const double2 swj = (Sw && own) ? Sw[row + t] : zero;
   const double2 sdj = delta ? Sd[row + t] : zero;
-  const bool has_w = swj.x != 0.0 || swj.y != 0.0;
-  const bool has_d = sdj.x != 0.0 || sdj.y != 0.0;
+  const bool has_w = has_load(swj);
+  const bool has_d = has_load(sdj);
   const double2 wj = own ? w[t] : zero;
   // this thread's product and output
   const int c = t / n, o = t - c * n;

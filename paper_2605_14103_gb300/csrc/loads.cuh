@@ -6,10 +6,17 @@
 
 namespace zbus {
 
+// Whether a slot carries a load (S != 0, NaN included), from the bits: a
+// comparison of doubles takes the FP64 pipe for 16 cycles of the SM a warp,
+// and the sweep steps made six of them per unknown beside some 35 operations.
+__device__ __forceinline__ bool has_load(double2 S) {
+  return ((__double_as_longlong(S.x) | __double_as_longlong(S.y)) << 1) != 0;
+}
+
 // conj(S / v) = conj(S) v / |v|^2; zero when the slot has no load.  The
 // multiply-adds are written out, so every kernel rounds alike.
 __device__ __forceinline__ double2 load_draw(double2 S, double2 v) {
-  if (S.x == 0.0 && S.y == 0.0) return make_double2(0.0, 0.0);
+  if (!has_load(S)) return make_double2(0.0, 0.0);
   const double inv = 1.0 / fma(v.x, v.x, v.y * v.y);
   return make_double2(fma(S.x, v.x, S.y * v.y) * inv, fma(S.x, v.y, -(S.y * v.x)) * inv);
 }
@@ -48,8 +55,8 @@ __device__ __forceinline__ void bus_injection_one(const double2* v, const double
   bool wye = false, delta = false;
 #pragma unroll
   for (int p = 0; p < 3; ++p) {
-    wye = wye || sw[p].x != 0.0 || sw[p].y != 0.0;
-    delta = delta || sd[p].x != 0.0 || sd[p].y != 0.0;
+    wye = wye || has_load(sw[p]);
+    delta = delta || has_load(sd[p]);
   }
   delta = delta && m == 3;
   if (wye && delta) {

@@ -417,9 +417,10 @@ k_split_pack(const double* __restrict__ Zr, const double* __restrict__ Zi, int n
 // between runs; no result depends on it.
 //
 // Bound by the FP64 pipe (about 34 operations an unknown at two a clock and
-// SM: 91 us for 4096 scenarios of 381 unknowns) and by the latencies between
-// the block's barriers: 156 us there, 203 before the voltages had a thread per
-// unknown and the slices one per four columns.
+// SM: 91 us for 4096 scenarios of 381 unknowns; 74 % busy) and by the
+// latencies between the block's barriers: 143 us there, 203 before the
+// voltages had a thread per unknown and the slices one per four columns, 156
+// before the tests for absent loads left the FP64 pipe.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double exact_double(long long x) {   // |x| < 2^51
   return __longlong_as_double(x + 0x4338000000000000ll) - 6755399441055744.0;
@@ -459,7 +460,7 @@ __device__ __forceinline__ void operand_of_bus(const SolveCtx& c, int b, int n, 
 }
 
 // Blocks of 256 threads an SM holds: at 2 the FP64 pipe waits (176 us a sweep
-// of 4096 scenarios of 381 unknowns against 156), at 4 the spills cost a few
+// of 4096 scenarios of 381 unknowns against 156, with comparisons on it), at 4 the spills cost a few
 // scenarios (92 us a sweep of 16 of 3069 unknowns against 76).
 constexpr int STEP_MIN = 3;
 
