@@ -596,7 +596,7 @@ def measure_gradient(net, Sw, Sd, n, args, flush, ws):
                      "mean_iters": float(ait.float().mean().item()),
                      "max_iters": int(ait.max().item()), "tol": GRAD_TOL}
     out["what"] = ("dL/dS_wye and dL/dS_delta of every scenario at its converged FP64 voltages "
-                   "(implicit-function adjoint; fp64: Z^T on the 3M contraction; tree: exact "
+                   "(implicit-function adjoint; fp64: Z^T on the forward contraction; tree: exact "
                    "Y^T residual and transposed tree sweep, one CTA per scenario)")
     return out
 

@@ -16,8 +16,8 @@
 // times the rate.
 //
 // Measured per sweep against the FP64 contraction (k_currents_f64 +
-// k_gemm3m_f64 + the stop test): 1000 scenarios of 3069 unknowns 66 -> 1.35 ms
-// (contraction 1.03), 4096 of 381 3.5 -> 0.24 ms (0.085).  Error of one map
+// k_gemm3m_f64 + the stop test): 1000 scenarios of 3069 unknowns 66 -> 1.32 ms
+// (contraction 1.03), 4096 of 381 3.5 -> 0.23 ms (0.085).  Error of one map
 // against extended precision, 102 to 2397 unknowns: 0.99 to 0.43 of the FP64
 // contraction's root mean square; of one adjoint sweep 0.70 to 0.28.
 //
