@@ -336,9 +336,14 @@ zbus_status run_group(Group* g, const std::vector<zbus_network>& nets, const std
   const double mtol = o.mismatch_tol > 0 ? o.mismatch_tol : 1e-6;
   for (auto net : nets) net->last_group = g;
   ZB_CHECK(group_reset(g, st));
-  for (size_t k = 0; k < nets.size(); ++k)
-    ZB_CHECK(group_admit(g, (int)k, 0, Bs[k], V0[k], Sw[k], Sd[k], st, false,
-                         o.fp32_start != 0));
+  // st waits for every lane whatever a launch says: the caller's buffers are in use
+  ZB_CHECK(group_fork(g, st));
+  zbus_status s = ZBUS_OK;
+  for (size_t k = 0; k < nets.size() && s == ZBUS_OK; ++k)
+    s = group_admit(g, (int)k, 0, Bs[k], V0[k], Sw[k], Sd[k], group_lane(g, k, st), false,
+                    o.fp32_start != 0);
+  ZB_CHECK(group_join(g, st));
+  ZB_CHECK(s);
   zbus_network pn = nets[0];
   if (o.profile == 1) {
     ZB_CHECK(ensure_profile(pn, max_iter));
@@ -351,10 +356,12 @@ zbus_status run_group(Group* g, const std::vector<zbus_network>& nets, const std
     ZB_CHECK(group_start(g, tol, max_iter, o.conv_rule, nullptr, 0, st));
     ZB_CHECK(group_run(g, st));
   }
-  for (size_t k = 0; k < nets.size(); ++k)
-    ZB_CHECK(group_collect(g, (int)k, 0, Bs[k], Vout[k], iters[k], conv[k], Sw[k], Sd[k], mtol,
-                           nullptr, o.max_correction, st));
-  return ZBUS_OK;
+  ZB_CHECK(group_fork(g, st));
+  for (size_t k = 0; k < nets.size() && s == ZBUS_OK; ++k)
+    s = group_collect(g, (int)k, 0, Bs[k], Vout[k], iters[k], conv[k], Sw[k], Sd[k], mtol,
+                      nullptr, o.max_correction, group_lane(g, k, st));
+  ZB_CHECK(group_join(g, st));
+  return s;
 }
 
 zbus_status check_device(zbus_network net) {

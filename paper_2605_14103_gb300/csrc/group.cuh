@@ -128,6 +128,10 @@ struct Group {
   std::vector<uint64_t> op_gen;  // operand generation of each item when built
   uint64_t tune_gen = 0;         // tile table generation when built
   cudaStream_t cap_stream = nullptr;
+  // the lanes beside the caller's stream (group_fork)
+  static constexpr int SIDE = 3;
+  cudaStream_t side[SIDE] = {};
+  cudaEvent_t forked = nullptr, joined[SIDE] = {};
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   // profile mode
@@ -136,6 +140,13 @@ struct Group {
   int prof_cap = 0;
   int prof_sweeps = 0;
 };
+
+// Lanes for launches of different items, which touch no common memory: what is
+// enqueued on group_lane(g, k, st) after group_fork runs after st's work so far,
+// and st's work after group_join after it.  A group of one item stays on st.
+zbus_status group_fork(Group* g, cudaStream_t st);
+cudaStream_t group_lane(const Group* g, size_t k, cudaStream_t st);
+zbus_status group_join(Group* g, cudaStream_t st);
 
 // lazy_ops: items whose tensor-core operands are not formed are built without
 // them (the serving cache forms them before the item's first admission and
