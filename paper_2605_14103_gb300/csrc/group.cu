@@ -2082,9 +2082,8 @@ void group_free(Group* g) {
 
 // The kernels of an item's admission and collection leave most SMs idle on a
 // feeder of a batch, and its correction graph is a chain of single blocks, so
-// four items at a time share the chip (16 feeders of
-// 50-800 buses 4.13 -> 3.31 ms, 3.25 with eight; two of 50 and 100 buses 412 ->
-// 365 us).
+// four items at a time share the chip (16 feeders of 50-800 buses 4.13 -> 3.31
+// ms, 3.25 with eight; two of 50 and 100 buses 412 -> 365 us).
 static int side_lanes(const Group* g) { return std::min((int)Group::SIDE, g->n_items - 1); }
 
 zbus_status group_fork(Group* g, cudaStream_t st) {
