@@ -252,6 +252,9 @@ typedef struct {
  * graph WHILE loop; each feeder's scenarios stop independently.  In FP64 the
  * feeders are solved one after another.  A network may appear at most once
  * per call.  Results equal those of zbus_solve on each feeder alone.
+ * Ordered like work on cuda_stream: what the call runs on streams of its own
+ * (admission and collection of different feeders) starts after the stream's
+ * earlier work and is waited for by its later work.
  */
 zbus_status zbus_solve_batched(const zbus_batch_item* items, int32_t n_items, double tol,
                                int32_t max_iter, const zbus_solve_opts* opts,
