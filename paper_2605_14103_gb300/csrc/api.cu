@@ -163,8 +163,10 @@ bool split_ready(zbus_network net, bool adjoint, cudaStream_t st) {
   if (ops->Z) return true;
   const std::string msg = g_last_error;
   const zbus_status s = adjoint
-                            ? split_pack(ops, net->ZrT, net->ZiT, net->n, net->n_pad, st)
-                            : split_pack(ops, net->Zr, net->Zi, net->n, net->n_pad, st);
+                            ? split_pack(ops, net->ZrT, net->ZiT, net->n, net->n_pad, net->part,
+                                         net->part_col, st)
+                            : split_pack(ops, net->Zr, net->Zi, net->n, net->n_pad, net->part,
+                                         net->part_col, st);
   if (s == ZBUS_OK) return true;
   g_last_error = msg;
   cudaGetLastError();
@@ -578,6 +580,8 @@ void zbus_network_destroy(zbus_network net) {
   cudaFree(net->Zi);
   cudaFree(net->Zs);
   cudaFree(net->Zt);
+  cudaFree(net->part);
+  cudaFree(net->part_col);
   cudaFree(net->csr_ptr);
   cudaFree(net->csr_col);
   cudaFree(net->csr_val);

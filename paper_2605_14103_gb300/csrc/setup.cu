@@ -541,6 +541,7 @@ zbus_status build_network(zbus_network net, int32_t n_total, int64_t nnz, const 
   ZB_CHECK(upload(&net->csr_ptr, lp, st));
   ZB_CHECK(upload(&net->csr_col, lc, st));
   ZB_CHECK(upload(&net->csr_val, lv, st));
+  if (split_size_ok(net->n_pad)) ZB_CHECK(split_parts(net, lp, lc, st));
   int32_t *d_sp = nullptr, *d_sc = nullptr;
   double2* d_sv = nullptr;
   zbus_status s = ZBUS_OK;

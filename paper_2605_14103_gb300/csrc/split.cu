@@ -1,5 +1,5 @@
 // The plain FP64 sweep (Sec. II-B) with its contraction Z i on the tensor
-// cores, without rounding: each operand is held as 55-bit fixed point with
+// cores, as sums of integers: each operand is held as 55-bit fixed point with
 // one power-of-two scale per row, cut into seven balanced 8-bit digits stored
 // in FP16 (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numerical
 // Algorithms 59, 2012).  A product of two digits is an integer of at most
@@ -7,9 +7,18 @@
 // adds those sums in 32-bit integers.  The complex product uses three real
 // ones (Re, Im and Re + Im, the sums formed as integers, so the scheme's
 // cancellations are exact), and the products of digits p and q are kept for
-// p + q <= 6: what is left out is about 2^-56 of the rows' largest entries
-// times the square root of n, below the rounding of an FP64 sum of n terms.  Every kept bit is an integer, so a result does not depend on the
+// p + q <= 6.  What the fixed point and the products left out cost is about
+// 2^-55 of a row's largest entry times the operand's largest, times the square
+// root of n.  Every kept bit is an integer, so a result does not depend on the
 // tile, the batch or the order of the sums.
+//
+// An FP64 sum's rounding goes with the sum of its terms' magnitudes instead,
+// so where a row's large entries meet small ones of the operand the fixed
+// point would be the less exact.  A 22nd product tells those rows: of the
+// leading digits of |Re| + |Im| (8 bits, rounded down), the sum of magnitudes
+// in units of the two scales.  Rows where it is below SPLIT_WEAK are formed in
+// FP64 by the step kernel, from the matrix and the operand themselves, over
+// the unknowns of the row's own part of the network.
 //
 // Why: this GPU does 1.25 TFLOP/s in FP64 and about 1.9 PFLOP/s in FP16; the
 // 28 digit products of 6 n^2 operations each are 168 n^2 operations at 1500
@@ -17,11 +26,9 @@
 //
 // Measured per sweep against the FP64 contraction (k_currents_f64 +
 // k_gemm3m_f64 + the stop test): 1000 scenarios of 3069 unknowns 66 -> 1.32 ms
-// (contraction 1.03), 4096 of 381 3.5 -> 0.23 ms (0.085).  Error of one map
-// against extended precision, 102 to 2397 unknowns: 0.99 to 0.43 of the FP64
-// contraction's root mean square; of one adjoint sweep 0.70 to 0.28.
+// (contraction 1.03), 4096 of 381 3.5 -> 0.23 ms (0.085).
 //
-// One sweep is two kernels: k_split_gemm (the 21 partial products of every
+// One sweep is two kernels: k_split_gemm (the 22 partial products of every
 // active scenario) and k_split_step (recombination, update, stop test, active
 // list and the operand of the next sweep, one block per scenario).
 #include <cuda_fp16.h>
@@ -41,6 +48,15 @@ namespace {
 using namespace tc;
 
 constexpr int GEMM_THREADS = 320;      // TMA, MMA and eight epilogue warps
+// Least sum of leading digits (unit 2^-14 of the product of the scales) of a
+// row that keeps its digit products: 1.5.  Root mean square error of a row
+// over that of the FP64 contraction, by this sum (99 and 255 unknowns; loads
+// and upstream gradients of one size, one bus of 100 or 10^4 times the others,
+// sizes over twelve decades): below 0.25 4 to 10^4, 0.5 to 0.75 1.0 to 2.4, 1 to
+// 1.25 1.0 to 1.5, 1.25 to 1.5 1.0 to 1.25, 1.5 to 2 0.8 to 1.15, above 2 at
+// most 0.95.  With loads of one size the rows below are those of the small
+// parts, a few buses behind a line of their own at the slack.
+constexpr int SPLIT_WEAK = 3 << 13;
 constexpr int EPI_WARPS = 8;
 constexpr int TMEM_COLS = 512;         // two accumulators of up to 256 columns
 constexpr int ACC_STRIDE = 256;
@@ -63,8 +79,8 @@ __device__ __forceinline__ void st_i8(int32_t* p, const int* v) {
 
 // ---------------------------------------------------------------------------
 // Work of the contraction: one item is the 128 x BN block (mt, nt) of one
-// partial product (c, d): component c (Re, Im, Re + Im) and digit weight d,
-// the sum over p <= d of X_p Z_{d-p}^T.  Items are listed from the longest
+// partial product (c, d): component c (Re, Im, Re + Im; 3, the magnitudes, has
+// one digit) and digit weight d, the sum over p <= d of X_p Z_{d-p}^T.  Items are listed from the longest
 // (d = 6) to the shortest and dealt to the blocks back and forth, so every
 // block gets about the same number of k-blocks.
 // ---------------------------------------------------------------------------
@@ -76,15 +92,16 @@ __device__ __forceinline__ SplitItem split_item(int g, int mtiles, int ntn) {
   const int per = mtiles * ntn;
   const int cls = g / per, t = g % per;
   SplitItem it;
-  it.d = SPLIT_S - 1 - cls / 3;
-  it.c = cls % 3;
+  it.d = cls < 3 * SPLIT_S ? SPLIT_S - 1 - cls / 3 : 0;
+  it.c = cls < 3 * SPLIT_S ? cls % 3 : 3;
   it.mt = t / ntn;
   it.nt = t % ntn;
   return it;
 }
 
 // k-blocks whose digit products sum exactly (to at most 2^24) in the FP32
-// accumulator: digits are at most 128, the first digit of Re + Im 256.
+// accumulator: digits are at most 128, the first digit of Re + Im and the
+// magnitudes 256.
 __device__ __forceinline__ int split_chunk(const SplitItem& it) {
   return (it.c < 2 ? 1024 : it.d > 0 ? 512 : 256) / BK;
 }
@@ -125,7 +142,7 @@ k_split_gemm(SolveCtx* __restrict__ ctx, const __grid_constant__ CUtensorMap tmX
   const int count = ctx->count;
   const int mtiles = (count + BM - 1) / BM;
   const int ntn = (n + BN - 1) / BN;
-  const int total = 3 * SPLIT_S * mtiles * ntn;
+  const int total = SPLIT_PLANES * mtiles * ntn;
   if ((int)blockIdx.x >= total) return;   // whole block, before any barrier
   const int rounds = (total + gridDim.x - 1) / gridDim.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -312,7 +329,7 @@ __device__ __forceinline__ long long fixed_point(double x, int e) {
   unsigned long long m = u & 0xFFFFFFFFFFFFFull;
   m = ex ? m | (1ull << 52) : m;
   // x = m 2^(max(ex, 1) - 1075)
-  const int sh = max(ex, 1) - 1075 + SPLIT_BITS - e;   // at most 1
+  const int sh = max(ex, 1) - 1075 + SPLIT_BITS - e;   // at most 2
   if (sh >= 0) {
     m <<= sh;
   } else if (sh < -55) {
@@ -325,7 +342,8 @@ __device__ __forceinline__ long long fixed_point(double x, int e) {
 
 // Slices of one row of n complex values, by all threads of the block: digit p
 // of component c of value(j) goes to plane c * 7 + p of out, `plane` halves
-// apart; a thread takes four columns of one component at a time.
+// apart, the leading digits of |Re| + |Im| to plane 21; a thread takes four
+// columns of one component at a time.
 template <typename Load>
 __device__ __forceinline__ void write_slices(Load value, int n, int K_pad, int e, __half* out,
                                              int64_t plane) {
@@ -334,14 +352,27 @@ __device__ __forceinline__ void write_slices(Load value, int n, int K_pad, int e
   for (int u = threadIdx.x; u < 3 * groups; u += blockDim.x) {
     const int c = u / groups, g = u - c * groups;
     long long y[4];
+    uint32_t mag[2] = {0x65006500u, 0x65006500u};   // 1280 + the magnitude's digit
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int j = g * 4 + i;
       const double2 v = j < n ? value(j) : make_double2(0.0, 0.0);
       y[i] = fixed_point(c == 1 ? v.y : v.x, e);
-      if (c == 2) y[i] += fixed_point(v.y, e);
+      if (c == 2) {
+        const long long im = fixed_point(v.y, e);
+        mag[i >> 1] += (uint32_t)((llabs(y[i]) + llabs(im)) >> (SPLIT_BITS - 7)) << (16 * (i & 1));
+        y[i] += im;
+      }
     }
     __half* dst = out + (int64_t)c * SPLIT_S * plane + g * 4;
+    if (c == 2) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const __half2 hv = __hsub2(*reinterpret_cast<const __half2*>(&mag[i]), bias);
+        mag[i] = *reinterpret_cast<const uint32_t*>(&hv);
+      }
+      *reinterpret_cast<uint2*>(dst + SPLIT_S * plane) = make_uint2(mag[0], mag[1]);
+    }
 #pragma unroll
     for (int p = SPLIT_S - 1; p >= 0; --p) {
       uint32_t w[2];
@@ -459,6 +490,58 @@ __device__ __forceinline__ void operand_of_bus(const SolveCtx& c, int b, int n, 
     if (p >= m) x[p] = make_double2(0.0, 0.0);
 }
 
+// The matrix in FP64 and its parts (SplitOps).
+struct SplitRows {
+  const double* Zr;
+  const double* Zi;
+  const int2* part;
+  const int32_t* part_col;
+  int n_pad;
+};
+
+// The weak rows of a warp (lane's: j0 + lane; `weak`, one bit each) in FP64,
+// four at a time, eight lanes a row over the unknowns of its part: in (re, im)
+// of their lanes.  x: the operand.  Columns without current cost no arithmetic.
+__device__ __noinline__ double2 weak_rows(unsigned weak, int j0, int n, const SplitRows& m,
+                                          const double2* x) {
+  const int lane = threadIdx.x & 31;
+  double2 mine = make_double2(0.0, 0.0);
+  while (weak) {
+    int bit[4], row = -1;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      bit[g] = __ffs(weak) - 1;   // -1: none left
+      weak &= weak - 1;
+      if (lane >> 3 == g && bit[g] >= 0) row = j0 + bit[g];
+    }
+    double2 a = make_double2(0.0, 0.0);
+    if (row >= 0) {
+      const int2 cols = __ldg(m.part + row);
+      const double* zr = m.Zr + (int64_t)row * m.n_pad;
+      const double* zi = m.Zi + (int64_t)row * m.n_pad;
+#pragma unroll 4
+      for (int t = cols.x + (lane & 7); t < cols.y; t += 8) {
+        const int k = __ldg(m.part_col + t);
+        if (!ZB_IN(k, n, 0x602u)) continue;
+        const double2 xk = x[k];
+        if (has_load(xk)) a = cfma(make_double2(__ldg(zr + k), __ldg(zi + k)), xk, a);
+      }
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+      a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+    }
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const double re = __shfl_sync(0xffffffffu, a.x, 8 * g);
+      const double im = __shfl_sync(0xffffffffu, a.y, 8 * g);
+      if (lane == bit[g]) mine = make_double2(re, im);
+    }
+  }
+  return mine;
+}
+
 // Blocks of 256 threads an SM holds: at 2 the FP64 pipe waits (176 us a sweep
 // of 4096 scenarios of 381 unknowns against 156, with comparisons on it), at 4 the spills cost a few
 // scenarios (92 us a sweep of 16 of 3069 unknowns against 76).
@@ -466,7 +549,7 @@ constexpr int STEP_MIN = 3;
 
 template <bool ADJ, bool FIRST>
 __global__ void __launch_bounds__(256, STEP_MIN)
-k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs,
+k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs, SplitRows m64,
              const double2* __restrict__ w, int n, int K_pad, int64_t rows,
              cudaGraphConditionalHandle h, int use_handle) {
   extern __shared__ double2 op[];   // [n] operand of the next sweep
@@ -487,20 +570,23 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs,
   const int count = c.count;
   for (int slot = blockIdx.x; slot < count; slot += gridDim.x) {
     const int b = list[slot];
-    const bool in = ZB_IN(b, c.B, 0x501u);
+    const bool in = ZB_IN(b, c.B, 0x601u);
     int out_slot = slot;
     double2* const V = c.V + (int64_t)(in ? b : 0) * n;
+    double2* const xop = c.xop + (int64_t)(in ? b : 0) * n;
     unsigned long long top = 0ull;       // largest |Re|, |Im| of the operand
     unsigned long long st2 = 0ull;       // largest squared step, bit pattern
     unsigned long long sth = 0ull;       // largest step whose square leaves the range
     double dsum = 0.0;
     const double xb = FIRST ? 0.0 : xs[slot];
     const double inv_s = ADJ ? 1.0 / c.gscale[in ? b : 0] : 0.0;
-    // voltages, a thread per unknown
+    // voltages, a thread per unknown (whole warps)
     if (in)
-      for (int j = tid; j < n; j += blockDim.x) {
+      for (int j0 = tid & ~31; j0 < n; j0 += blockDim.x) {
+        const bool own = j0 + (tid & 31) < n;
+        const int j = own ? j0 + (tid & 31) : n - 1;
         if (FIRST) {
-          op[j] = V[j];
+          if (own) op[j] = V[j];
           continue;
         }
         const int32_t* D = c.D + (int64_t)slot * ld + j;
@@ -510,9 +596,10 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs,
         for (int q = 0; q < 3; ++q)
 #pragma unroll
           for (int d = 0; d < SPLIT_S; ++d) t[q][d] = D[(q * SPLIT_S + d) * plane];
+        const bool low = D[3 * SPLIT_S * plane] < SPLIT_WEAK;
         const double2 vo = V[j];
         const double2 wj = ADJ ? make_double2(0.0, 0.0) : w[j];
-        const double s = zs[j] * xb;
+        double s = zs[j] * xb;
         long long hi[3], lo[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
@@ -520,8 +607,20 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs,
                   ((long long)t[q][2] << 8) + t[q][3];
           lo[q] = ((long long)t[q][4] << 16) + ((long long)t[q][5] << 8) + t[q][6];
         }
-        const double re = recombine(hi[0] - hi[1], lo[0] - lo[1]);
-        const double im = recombine(hi[2] - hi[0] - hi[1], lo[2] - lo[0] - lo[1]);
+        double re = recombine(hi[0] - hi[1], lo[0] - lo[1]);
+        double im = recombine(hi[2] - hi[0] - hi[1], lo[2] - lo[0] - lo[1]);
+        // a scale of zero (no current at all) or one that is not a number
+        // gives every row its value
+        const unsigned weak = __ballot_sync(0xffffffffu, own && low && xb > 0.0);
+        if (weak) {
+          const double2 f = weak_rows(weak, j0, n, m64, xop);
+          if (weak >> (tid & 31) & 1) {
+            re = f.x;
+            im = f.y;
+            s = 1.0;
+          }
+        }
+        if (!own) continue;
         const double2 v = make_double2(fma(re, s, wj.x), fma(im, s, wj.y));
         V[j] = v;
         op[j] = v;
@@ -600,13 +699,17 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs,
     const int e = bad ? 0 : row_exponent(top);
     __half* out = reinterpret_cast<__half*>(c.X) + (int64_t)out_slot * K_pad;
     const int64_t plane = rows * K_pad;
+    if (in)
+      for (int j = tid; j < n; j += blockDim.x) xop[j] = op[j];
     if (bad) {
       write_slices([&](int) { return make_double2(0.0, 0.0); }, n, K_pad, 0, out, plane);
     } else {
       write_slices([&](int j) { return op[j]; }, n, K_pad, e, out, plane);
     }
     if (tid == 0)
-      xs_out[out_slot] = bad ? __longlong_as_double(0x7FF8000000000000ll) : ldexp(1.0, e - 31);
+      xs_out[out_slot] = bad    ? __longlong_as_double(0x7FF8000000000000ll)
+                         : top ? ldexp(1.0, e - 31)
+                               : 0.0;
     __syncthreads();
   }
   if (FIRST) return;
@@ -640,7 +743,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// Planes [21][rows][K_pad] of FP16 as a 3D tensor, boxes of 64 x box_rows;
+// Planes [22][rows][K_pad] of FP16 as a 3D tensor, boxes of 64 x box_rows;
 // rows past the end read as zero.
 zbus_status make_map(CUtensorMap* map, const void* base, int K_pad, int64_t rows, int box_rows) {
   auto fn = encode_fn();
@@ -699,7 +802,8 @@ int step_grid(int64_t batch) {
 
 size_t split_scratch_bytes(int n, int64_t rows) {
   return a256((size_t)SPLIT_PLANES * rows * split_kpad(n) * 2) +
-         a256((size_t)SPLIT_PLANES * rows * split_ld(n) * 4) + a256((size_t)rows * 2 * 8) +
+         a256((size_t)SPLIT_PLANES * rows * split_ld(n) * 4) +
+         a256((size_t)rows * n * sizeof(double2)) + a256((size_t)rows * 2 * 8) +
          a256((size_t)rows * 4);
 }
 
@@ -710,15 +814,58 @@ zbus_status split_scratch_bind(SplitScratch* s, void* base, int n, int64_t rows)
   p += a256((size_t)SPLIT_PLANES * rows * split_kpad(n) * 2);
   s->D = (int32_t*)p;
   p += a256((size_t)SPLIT_PLANES * rows * split_ld(n) * 4);
+  s->xop = (double2*)p;
+  p += a256((size_t)rows * n * sizeof(double2));
   s->xs = (double*)p;
   p += a256((size_t)rows * 2 * 8);
   s->list2 = (int32_t*)p;
   return make_map(&s->map, s->X, split_kpad(n), rows, BM);
 }
 
+zbus_status split_parts(zbus_network net, const std::vector<int32_t>& ptr,
+                        const std::vector<int32_t>& col, cudaStream_t st) {
+  const int n = net->n;
+  std::vector<int32_t> root(n);
+  for (int i = 0; i < n; ++i) root[i] = i;
+  auto find = [&](int i) {
+    while (root[i] != i) i = root[i] = root[root[i]];
+    return i;
+  };
+  for (int i = 0; i < n; ++i)
+    for (int t = ptr[i]; t < ptr[i + 1]; ++t) {
+      const int a = find(i), b = find(col[t]);
+      root[std::max(a, b)] = std::min(a, b);
+    }
+  std::vector<int32_t> order(n);
+  for (int i = 0; i < n; ++i) {
+    root[i] = find(i);
+    order[i] = i;
+  }
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return root[a] < root[b]; });
+  std::vector<int2> range(n);
+  for (int i = 0, e = 0; i < n; i = e) {
+    for (e = i; e < n && root[order[e]] == root[order[i]]; ++e) {
+    }
+    for (int t = i; t < e; ++t) range[order[t]] = make_int2(i, e);
+  }
+  ZB_CUDA(cudaMalloc((void**)&net->part, (size_t)n * sizeof(int2)));
+  ZB_CUDA(cudaMalloc((void**)&net->part_col, (size_t)n * sizeof(int32_t)));
+  ZB_CUDA(cudaMemcpyAsync(net->part, range.data(), (size_t)n * sizeof(int2),
+                          cudaMemcpyHostToDevice, st));
+  ZB_CUDA(cudaMemcpyAsync(net->part_col, order.data(), (size_t)n * sizeof(int32_t),
+                          cudaMemcpyHostToDevice, st));
+  ZB_CUDA(cudaStreamSynchronize(st));
+  return ZBUS_OK;
+}
+
 zbus_status split_pack(SplitOps* ops, const double* Zr, const double* Zi, int n, int n_pad,
-                       cudaStream_t st) {
+                       const int2* part, const int32_t* part_col, cudaStream_t st) {
   if (ops->Z) return ZBUS_OK;
+  ops->Zr = Zr;
+  ops->Zi = Zi;
+  ops->n_pad = n_pad;
+  ops->part = part;
+  ops->part_col = part_col;
   const int K = split_kpad(n);
   // N-tile: 192 or 256 outputs, whichever leaves less of the last tile idle
   ops->BN = round_up(n, 192) < round_up(n, 256) ? 192 : 256;
@@ -750,6 +897,7 @@ void split_fill_ctx(SolveCtx* h, const SplitScratch& s) {
   h->X = s.X;
   h->D = s.D;
   h->xs = s.xs;
+  h->xop = s.xop;
   h->list2 = s.list2;
   h->next = 0;
   h->done = 0;
@@ -764,14 +912,15 @@ zbus_status launch_split_gemm(SolveCtx* ctx, const SplitScratch& s, const SplitO
 namespace {
 
 template <bool ADJ, bool FIRST>
-void launch_step(SolveCtx* ctx, const double* zs, const double2* w, int n, int64_t batch,
+void launch_step(SolveCtx* ctx, const SplitOps& ops, const double2* w, int n, int64_t batch,
                  int64_t rows, cudaGraphConditionalHandle h, bool use_handle, cudaStream_t st) {
+  const SplitRows m64 = {ops.Zr, ops.Zi, ops.part, ops.part_col, ops.n_pad};
   const size_t smem = (size_t)n * sizeof(double2);
   if (smem > 32 * 1024)
     cudaFuncSetAttribute(k_split_step<ADJ, FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
   k_split_step<ADJ, FIRST><<<step_grid(batch), step_threads(n), smem, st>>>(
-      ctx, zs, w, n, split_kpad(n), rows, h, use_handle ? 1 : 0);
+      ctx, ops.zs, m64, w, n, split_kpad(n), rows, h, use_handle ? 1 : 0);
 }
 
 }  // namespace
@@ -779,18 +928,18 @@ void launch_step(SolveCtx* ctx, const double* zs, const double2* w, int n, int64
 void launch_split_first(SolveCtx* ctx, int n, int64_t batch, int64_t rows, bool adjoint,
                         cudaStream_t st) {
   if (adjoint)
-    launch_step<true, true>(ctx, nullptr, nullptr, n, batch, rows, 0, false, st);
+    launch_step<true, true>(ctx, SplitOps(), nullptr, n, batch, rows, 0, false, st);
   else
-    launch_step<false, true>(ctx, nullptr, nullptr, n, batch, rows, 0, false, st);
+    launch_step<false, true>(ctx, SplitOps(), nullptr, n, batch, rows, 0, false, st);
 }
 
 void launch_split_step(SolveCtx* ctx, const SplitOps& ops, const double2* w, int n, int64_t batch,
                        int64_t rows, bool adjoint, cudaGraphConditionalHandle h, bool use_handle,
                        cudaStream_t st) {
   if (adjoint)
-    launch_step<true, false>(ctx, ops.zs, nullptr, n, batch, rows, h, use_handle, st);
+    launch_step<true, false>(ctx, ops, nullptr, n, batch, rows, h, use_handle, st);
   else
-    launch_step<false, false>(ctx, ops.zs, w, n, batch, rows, h, use_handle, st);
+    launch_step<false, false>(ctx, ops, w, n, batch, rows, h, use_handle, st);
 }
 
 ZB_CHECK_WORD_ACCESSOR(check_word_split)

@@ -6,12 +6,14 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "zbus_internal.cuh"
 
 namespace zbus {
 
 constexpr int SPLIT_S = 7;                        // slices of 8 bits
-constexpr int SPLIT_PLANES = 3 * SPLIT_S;         // Re, Im, Re + Im
+constexpr int SPLIT_PLANES = 3 * SPLIT_S + 1;     // Re, Im, Re + Im; magnitudes
 constexpr int SPLIT_BITS = 55;                    // |fixed-point Re, Im| <= 2^55
 // Padded unknowns the path takes.  Below, k_solve_fused_f64 runs a whole small
 // solve in one launch.  From there on the path is the faster one at every
@@ -32,12 +34,19 @@ inline size_t split_ops_bytes(int n) {
   return (size_t)SPLIT_PLANES * n * split_kpad(n) * 2 + (size_t)n * sizeof(double);
 }
 
+// The independent parts of a network (unknowns that its admittances join; Z is
+// zero between two parts), from the sparse rows of Y_LL (host): the unknowns
+// part by part, and each unknown's range of that list.
+zbus_status split_parts(zbus_network net, const std::vector<int32_t>& ptr,
+                        const std::vector<int32_t>& col, cudaStream_t st);
+
 size_t split_scratch_bytes(int n, int64_t rows);
 zbus_status split_scratch_bind(SplitScratch* s, void* base, int n, int64_t rows);
 
-// The slices of a matrix given by its 3M copies (row-major [n_pad][n_pad]).
+// The slices of a matrix given by its 3M copies (row-major [n_pad][n_pad],
+// read by the sweeps too) and its parts (split_parts).
 zbus_status split_pack(SplitOps* ops, const double* Zr, const double* Zi, int n, int n_pad,
-                       cudaStream_t st);
+                       const int2* part, const int32_t* part_col, cudaStream_t st);
 void split_release(SplitOps* ops);
 
 // First operand of a solve (after k_init / k_adj_init wrote the context, its

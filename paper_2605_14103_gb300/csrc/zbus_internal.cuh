@@ -138,6 +138,7 @@ struct SolveCtx {
   void* X;
   int32_t* D;
   double* xs;
+  double2* xop;           // [B][n] the operand itself
   int32_t* list2;
   int32_t next;
   int32_t done;
@@ -145,8 +146,13 @@ struct SolveCtx {
 
 // Slices of a matrix for the plain method's tensor-core contraction.
 struct SplitOps {
-  void* Z = nullptr;         // [21][n][K_pad] FP16 digits
+  void* Z = nullptr;         // [22][n][K_pad] FP16 digits
   double* zs = nullptr;      // [n] row scales
+  const double* Zr = nullptr;   // [n][n_pad] the matrix itself
+  const double* Zi = nullptr;
+  int n_pad = 0;
+  const int2* part = nullptr;         // [n] range of an unknown's part in part_col
+  const int32_t* part_col = nullptr;  // [n] unknowns, part by part
   int BN = 0;                // N-tile
   CUtensorMap map;           // of Z
 };
@@ -154,8 +160,9 @@ struct SplitOps {
 // Scratch of `rows` active scenarios, in a caller-provided buffer.
 struct SplitScratch {
   int64_t rows = 0;
-  void* X = nullptr;         // [21][rows][K_pad] FP16 slices of the operand
-  int32_t* D = nullptr;      // [21][rows][ld] exact partial products
+  void* X = nullptr;         // [22][rows][K_pad] FP16 slices of the operand
+  int32_t* D = nullptr;      // [22][rows][ld] exact partial products
+  double2* xop = nullptr;    // [rows][n] the operand, by scenario
   double* xs = nullptr;      // [2][rows] operand scales, by sweep parity
   int32_t* list2 = nullptr;  // [rows] second active list
   CUtensorMap map;           // of X
@@ -248,6 +255,8 @@ struct zbus_network_s {
   double* Zi = nullptr;
   double* Zs = nullptr;      // Zr + Zi
   double* Zt = nullptr;      // small feeders: the three transposed, [3][n_pad][n_pad]
+  int2* part = nullptr;         // independent parts (split_parts), of the sizes the
+  int32_t* part_col = nullptr;  // tensor-core path takes
   int32_t* csr_ptr = nullptr;   // Y_LL rows (n + 1)
   int32_t* csr_col = nullptr;
   double2* csr_val = nullptr;
