@@ -23,6 +23,7 @@
 #include "df.cuh"
 #include "group.cuh"
 #include "loads.cuh"
+#include "split.cuh"
 #include "tc_ptx.cuh"
 
 namespace zbus {
@@ -660,7 +661,8 @@ k_contract_group(GroupState* __restrict__ gs, const ItemDesc* __restrict__ items
       const ItemDesc& it = items[k];
       const int buf = i & 1;
       const uint32_t use = (uint32_t)(i >> 1);
-      const bool ok = mbar_wait(&tfull[buf], use & 1, wait_ns);
+      // the warp goes on, or gives up, as one: its loads need every lane
+      const bool ok = __all_sync(0xffffffffu, mbar_wait(&tfull[buf], use & 1, wait_ns));
       tc_fence_after();
       if (!ok) {
         if (lane == 0) atomicCAS(&gs->err, 0, 103);
@@ -2632,6 +2634,7 @@ extern "C" zbus_status zbus_checked_set_wait(uint64_t wait_ns) {
 #ifdef ZBUS_CHECKED
   zbus::set_error("");
   cudaError_t e = cudaMemcpyToSymbol(zbus::g_tc_wait_ns, &wait_ns, sizeof(wait_ns));
+  if (e == cudaSuccess) e = zbus::split_set_wait(wait_ns);
   if (e != cudaSuccess)
     return zbus::cuda_fail(e, "cudaMemcpyToSymbol(wait limit)", __FILE__, __LINE__);
   return ZBUS_OK;

@@ -62,6 +62,14 @@ constexpr int TMEM_COLS = 512;         // two accumulators of up to 256 columns
 constexpr int ACC_STRIDE = 256;
 constexpr unsigned long long SPLIT_DRAIN_NS = 2000000000ull;
 
+#ifdef ZBUS_CHECKED
+// checked build: zbus_checked_set_wait lowers the limit of the pipeline's waits
+__device__ unsigned long long g_split_wait_ns = WAIT_NS;
+__device__ __forceinline__ unsigned long long split_wait_ns() { return g_split_wait_ns; }
+#else
+__device__ __forceinline__ unsigned long long split_wait_ns() { return WAIT_NS; }
+#endif
+
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar,
                                             int x, int y, int z) {
   asm volatile(
@@ -145,6 +153,7 @@ k_split_gemm(SolveCtx* __restrict__ ctx, const __grid_constant__ CUtensorMap tmX
   const int total = SPLIT_PLANES * mtiles * ntn;
   if ((int)blockIdx.x >= total) return;   // whole block, before any barrier
   const int rounds = (total + gridDim.x - 1) / gridDim.x;
+  const unsigned long long wait_ns = split_wait_ns();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
@@ -184,7 +193,7 @@ k_split_gemm(SolveCtx* __restrict__ ctx, const __grid_constant__ CUtensorMap tmX
           for (int kb = 0; kb < num_kb; ++kb) {
             const int s = kc % STAGES;
             const uint32_t round = kc / STAGES;
-            if (!mbar_wait(&empty[s], (round & 1) ^ 1)) {
+            if (!mbar_wait(&empty[s], (round & 1) ^ 1, wait_ns)) {
               atomicCAS(&ctx->err, 0, 111);
               ok = false;
               break;
@@ -219,7 +228,7 @@ k_split_gemm(SolveCtx* __restrict__ ctx, const __grid_constant__ CUtensorMap tmX
         const int blocks = (it.d + 1) * num_kb, chunk = split_chunk(it);
         for (int b0 = 0; b0 < blocks && ok; b0 += chunk, ++ch) {
           const int buf = ch & 1;
-          if (!mbar_wait(&tempty[buf], ((ch >> 1) & 1) ^ 1)) {
+          if (!mbar_wait(&tempty[buf], ((ch >> 1) & 1) ^ 1, wait_ns)) {
             atomicCAS(&ctx->err, 0, 114);
             ok = false;
             break;
@@ -229,7 +238,7 @@ k_split_gemm(SolveCtx* __restrict__ ctx, const __grid_constant__ CUtensorMap tmX
           const int b1 = min(blocks, b0 + chunk);
           for (int b = b0; b < b1; ++b, ++kc) {
             const int s = kc % STAGES;
-            if (!mbar_wait(&full[s], (kc / STAGES) & 1)) {
+            if (!mbar_wait(&full[s], (kc / STAGES) & 1, wait_ns)) {
               atomicCAS(&ctx->err, 0, 112);
               ok = false;
               break;
@@ -269,7 +278,8 @@ k_split_gemm(SolveCtx* __restrict__ ctx, const __grid_constant__ CUtensorMap tmX
       for (int t = 0; t < HN; ++t) acc[t] = 0;
       for (int b0 = 0; b0 < blocks; b0 += chunk, ++ch) {
         const int buf = ch & 1;
-        ok = mbar_wait(&tfull[buf], (ch >> 1) & 1);
+        // the warp goes on, or gives up, as one: its loads need every lane
+        ok = __all_sync(0xffffffffu, mbar_wait(&tfull[buf], (ch >> 1) & 1, wait_ns));
         tc_fence_after();
         if (!ok) {
           if (lane == 0) atomicCAS(&ctx->err, 0, 113);
@@ -943,5 +953,14 @@ void launch_split_step(SolveCtx* ctx, const SplitOps& ops, const double2* w, int
 }
 
 ZB_CHECK_WORD_ACCESSOR(check_word_split)
+
+cudaError_t split_set_wait(uint64_t wait_ns) {
+#ifdef ZBUS_CHECKED
+  return cudaMemcpyToSymbol(g_split_wait_ns, &wait_ns, sizeof(wait_ns));
+#else
+  (void)wait_ns;
+  return cudaErrorNotSupported;
+#endif
+}
 
 }  // namespace zbus

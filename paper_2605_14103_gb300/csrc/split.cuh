@@ -49,6 +49,9 @@ zbus_status split_pack(SplitOps* ops, const double* Zr, const double* Zi, int n,
                        const int2* part, const int32_t* part_col, cudaStream_t st);
 void split_release(SplitOps* ops);
 
+// The checked build's wait limit (zbus_checked_set_wait).
+cudaError_t split_set_wait(uint64_t wait_ns);
+
 // First operand of a solve (after k_init / k_adj_init wrote the context, its
 // list and the start), and one sweep of up to `batch` scenarios: contraction,
 // then update, stop test, active list and the next operand.  adjoint: the
