@@ -437,8 +437,8 @@ zbus_status zbus_last_profile(zbus_network net, int32_t max_n, float* ms, int32_
  * property of this library's interface.
  *
  * It calls no cudaMalloc, cudaFree or allocating library routine: its scratch
- * (solve context, active list, per-tile partials, contraction operands) lives
- * in one static 16 MiB device array.  zbus_network_create loads that array on
+ * (active list, per-tile partials, contraction operands) lives in one static
+ * 16 MiB device array.  zbus_network_create loads that array on
  * its device and looks up its address (with that device current), so every
  * device on which a network was created holds the 16 MiB from then until the
  * process exits, and this call itself loads nothing.  The network must exist

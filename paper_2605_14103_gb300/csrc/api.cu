@@ -62,8 +62,9 @@ int max_ntn(const zbus_network net) {
 
 int k_pad_tc(const zbus_network net) { return round_up(2 * net->n, 64); }
 
-// Scratch of one solve: context, active list, per-tile partials, the FP64
-// contraction operands and the low-precision residual rows.
+// Scratch of one solve: active list, per-tile partials, the FP64 contraction
+// operands and the low-precision residual rows.  (The context stays with the
+// network: zbus_last_device_status reads it after the scratch has grown.)
 struct WsLayout {
   size_t list, keep, part, iop, R, rinv, mm, v4, swf, sdf, st, amax, mt, sit, sconv, total;
 };
@@ -73,7 +74,7 @@ WsLayout workspace_layout(const zbus_network net, int64_t B) {
   // 128-scenario tile of the tensor-core contraction
   const size_t Bp = (size_t)round_up((int)B, 128);
   WsLayout L;
-  size_t o = align256(sizeof(SolveCtx));
+  size_t o = 0;
   L.list = o;
   o += align256((size_t)B * sizeof(int32_t));
   L.keep = o;
@@ -133,7 +134,7 @@ zbus_status ensure_workspace(zbus_network net, int64_t B) {
   ws.bytes = L.total;
   ws.cap_B = B;
   ws.cap_Bp = round_up((int)B, 128);
-  ws.ctx = (SolveCtx*)p;
+  ws.ctx = net->ctx;
   ws.list = (int32_t*)(p + L.list);
   ws.keep = (uint8_t*)(p + L.keep);
   ws.part = (double*)(p + L.part);
@@ -336,7 +337,10 @@ zbus_status run_group(Group* g, const std::vector<zbus_network>& nets, const std
                       const std::vector<int32_t*>& iters, const std::vector<uint8_t*>& conv,
                       double tol, int32_t max_iter, const zbus_solve_opts& o, cudaStream_t st) {
   const double mtol = o.mismatch_tol > 0 ? o.mismatch_tol : 1e-6;
-  for (auto net : nets) net->last_group = g;
+  for (auto net : nets) {
+    net->last_group = g;
+    net->last_ctx = nullptr;
+  }
   ZB_CHECK(group_reset(g, st));
   // st waits for every lane whatever a launch says: the caller's buffers are in use
   ZB_CHECK(group_fork(g, st));
@@ -568,6 +572,7 @@ void zbus_network_destroy(zbus_network net) {
   }
   cudaFree(net->prof.d_hist);
   cudaFree(net->ws.base);
+  cudaFree(net->ctx);
   free_mixed(net);
   phased_free(net);
   free_adjoint(net);

@@ -9,7 +9,8 @@
 // at start-up (zbus_network_create allocates) and then calls this entry point,
 // which calls no cudaMalloc, cudaFree or allocating library routine.
 //
-// The scratch array is STATIC_SCRATCH_BYTES (16 MiB).  The CUDA runtime loads
+// The solve's context is the network's own (so each network keeps its error
+// word).  The scratch array is STATIC_SCRATCH_BYTES (16 MiB).  The CUDA runtime loads
 // it on a device lazily, when its address is first asked for; so that this
 // never happens inside a call that must not allocate, zbus_network_create
 // asks for it (noalloc_prepare), and every device on which a network was
@@ -88,9 +89,9 @@ extern "C" zbus_status zbus_solve_noalloc(zbus_network net, int64_t B, const dou
   if (S_delta && !net->bus_aligned)
     return fail(ZBUS_ERR_ARG, "delta loads need three unknowns per bus (n % 3 == 0)");
 
-  // scratch layout: context | active list | keep marks | per-tile partials | 3M operands
+  // scratch layout: active list | keep marks | per-tile partials | 3M operands
   const int ntn = net->n_pad / F64_BN;
-  const size_t o_list = a256(sizeof(SolveCtx));
+  const size_t o_list = 0;
   const size_t o_keep = o_list + a256((size_t)B * sizeof(int32_t));
   const size_t o_part = o_keep + a256((size_t)B);
   const size_t o_iop = o_part + a256((size_t)B * ntn * 2 * sizeof(double));
@@ -135,7 +136,7 @@ extern "C" zbus_status zbus_solve_noalloc(zbus_network net, int64_t B, const dou
   h.max_iter = max_iter;
   h.rule = conv_rule;
   h.ntn = ntn;
-  SolveCtx* ctx = (SolveCtx*)p;
+  SolveCtx* ctx = net->ctx + 1;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   // zbus_last_device_status must not report the error word of an earlier
   // mixed-precision solve
@@ -149,15 +150,14 @@ extern "C" zbus_status zbus_solve_noalloc(zbus_network net, int64_t B, const dou
     // the contraction on the tensor cores, as zbus_solve: its scratch takes
     // more bytes per scenario, so the batch runs in passes of the scenarios
     // that fit (independent of each other: the same bits)
-    const size_t fixed = a256(sizeof(SolveCtx));
     const size_t per = split_scratch_bytes(net->n, 256) / 256 + sizeof(int32_t);
-    const int64_t rows = std::min<int64_t>(B, (int64_t)((STATIC_SCRATCH_BYTES - fixed - 4096) / per));
+    const int64_t rows = std::min<int64_t>(B, (int64_t)((STATIC_SCRATCH_BYTES - 4096) / per));
     if (rows >= 1) {
       SplitScratch scratch;
-      ZB_CHECK(split_scratch_bind(&scratch, p + fixed + a256((size_t)rows * sizeof(int32_t)),
-                                  net->n, rows));
+      ZB_CHECK(split_scratch_bind(&scratch, p + a256((size_t)rows * sizeof(int32_t)), net->n,
+                                  rows));
       net->last_ctx = ctx;
-      h.list = (int32_t*)(p + fixed);
+      h.list = (int32_t*)p;
       split_fill_ctx(&h, scratch);
       for (int64_t b0 = 0; b0 < B; b0 += rows) {
         const int64_t Bk = std::min(rows, B - b0);

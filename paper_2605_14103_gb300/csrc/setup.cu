@@ -536,6 +536,7 @@ zbus_status build_network(zbus_network net, int32_t n_total, int64_t nnz, const 
     ZB_CHECK(build_tree(net, bp, bc, bv, st));
   }
 
+  ZB_CUDA(cudaMalloc((void**)&net->ctx, 2 * sizeof(SolveCtx)));
   ZB_CUDA(cudaMalloc((void**)&net->w, n * sizeof(double2)));
   ZB_CUDA(cudaMalloc((void**)&net->ys, n * sizeof(double2)));
   ZB_CHECK(upload(&net->csr_ptr, lp, st));

@@ -335,7 +335,10 @@ struct zbus_network_s {
   zbus::SplitOps split_zt;
   zbus::SplitScratch split;
   void* split_base = nullptr;
-  const zbus::SolveCtx* last_ctx = nullptr;   // context of the last such solve (error word)
+  // contexts of zbus_solve / zbus_solve_adjoint and of zbus_solve_noalloc, and
+  // that of the last such solve with device-side waits (error word)
+  zbus::SolveCtx* ctx = nullptr;   // [2]
+  const zbus::SolveCtx* last_ctx = nullptr;
 };
 
 namespace zbus {
