@@ -174,11 +174,27 @@ bool split_ready(zbus_network net, bool adjoint, cudaStream_t st) {
   return false;
 }
 
+// The checked build's stand-in for a device too full for an allocation of more
+// than so many bytes.
+static bool split_alloc_fits(size_t bytes) {
+#ifdef ZBUS_CHECKED
+  const char* e = std::getenv("ZBUS_CHECKED_SPLIT_BYTES");
+  return !e || bytes <= std::strtoull(e, nullptr, 10);
+#else
+  (void)bytes;
+  return true;
+#endif
+}
+
 int64_t split_rows(zbus_network net, int64_t B) {
   const size_t per = split_scratch_bytes(net->n, 128) / 128;
   const int64_t most = std::max<int64_t>(128, (int64_t)(SPLIT_SCRATCH_MAX / per) / 128 * 128);
-  const int64_t want = std::min(most, (B + 127) / 128 * 128);
-  if (net->split.rows >= want) return net->split.rows;
+  int64_t want = std::min(most, (B + 127) / 128 * 128);
+  // a size asked for before and not to be had is not tried at every call
+  // (zbus_network_reserve tries it again)
+  if (net->split.rows >= want || (net->split.rows > 0 && net->split_asked >= want))
+    return net->split.rows;
+  net->split_asked = want;
   if (net->split_base) {
     if (cudaDeviceSynchronize() != cudaSuccess) return 0;
     drop_graphs(net);
@@ -186,10 +202,13 @@ int64_t split_rows(zbus_network net, int64_t B) {
     net->split_base = nullptr;
     net->split = SplitScratch();
   }
+  // on a device too full for all of it, half the scenarios a pass, and so on
   void* base = nullptr;
-  if (cudaMalloc(&base, split_scratch_bytes(net->n, want)) != cudaSuccess) {
+  while (!split_alloc_fits(split_scratch_bytes(net->n, want)) ||
+         cudaMalloc(&base, split_scratch_bytes(net->n, want)) != cudaSuccess) {
     cudaGetLastError();
-    return 0;
+    if (want <= 128) return 0;
+    want = (want / 2 + 127) / 128 * 128;
   }
   if (split_scratch_bind(&net->split, base, net->n, want) != ZBUS_OK) {
     cudaFree(base);
@@ -643,7 +662,10 @@ zbus_status zbus_network_reserve(zbus_network net, int64_t B, int32_t precision)
   ZB_CHECK(check_device(net));
   ZB_CHECK(ensure_workspace(net, B));
   ZB_CHECK(ensure_3m(net, nullptr));
-  if (precision == ZBUS_FP64 && split_ready(net, false, nullptr)) split_rows(net, B);
+  if (precision == ZBUS_FP64 && split_ready(net, false, nullptr)) {
+    net->split_asked = 0;
+    split_rows(net, B);
+  }
   if (precision == ZBUS_TREE_SWEEP) ZB_CHECK(prepare_tree(net, nullptr));
   else if (precision != ZBUS_FP64) ZB_CHECK(prepare_mixed(net, precision, nullptr));
   return ZBUS_OK;

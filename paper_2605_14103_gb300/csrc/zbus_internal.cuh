@@ -335,6 +335,7 @@ struct zbus_network_s {
   zbus::SplitOps split_zt;
   zbus::SplitScratch split;
   void* split_base = nullptr;
+  int64_t split_asked = 0;   // largest number of scenarios asked for
   // contexts of zbus_solve / zbus_solve_adjoint and of zbus_solve_noalloc, and
   // that of the last such solve with device-side waits (error word)
   zbus::SolveCtx* ctx = nullptr;   // [2]
