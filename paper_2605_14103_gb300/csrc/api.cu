@@ -186,6 +186,13 @@ static bool split_alloc_fits(size_t bytes) {
 #endif
 }
 
+void split_drop_scratch(zbus_network net) {
+  drop_graphs(net);
+  cudaFree(net->split_base);
+  net->split_base = nullptr;
+  net->split = SplitScratch();
+}
+
 int64_t split_rows(zbus_network net, int64_t B) {
   const size_t per = split_scratch_bytes(net->n, 128) / 128;
   const int64_t most = std::max<int64_t>(128, (int64_t)(SPLIT_SCRATCH_MAX / per) / 128 * 128);
@@ -197,10 +204,7 @@ int64_t split_rows(zbus_network net, int64_t B) {
   net->split_asked = want;
   if (net->split_base) {
     if (cudaDeviceSynchronize() != cudaSuccess) return 0;
-    drop_graphs(net);
-    cudaFree(net->split_base);
-    net->split_base = nullptr;
-    net->split = SplitScratch();
+    split_drop_scratch(net);
   }
   // on a device too full for all of it, half the scenarios a pass, and so on
   void* base = nullptr;

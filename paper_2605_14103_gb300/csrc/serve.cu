@@ -189,8 +189,8 @@ extern "C" zbus_status zbus_serve(const zbus_serve_config* cfg, zbus_network* po
                               "operands of the largest feeder (" +
                                   std::to_string(per_slot * 128 + peak_one) + " bytes)");
   const size_t ops_budget = budget - (size_t)per_slot * cap;
-  // the slices the plain method keeps of each Z are no part of the cache:
-  // they stay only where they fit beside all of it
+  // the slices the plain method keeps of each Z and the scratch of its sweeps
+  // are no part of the cache: they stay only where they fit beside all of it
   {
     size_t all = 0, most_form = 0, slices = 0;
     for (auto net : nets) {
@@ -198,11 +198,12 @@ extern "C" zbus_status zbus_serve(const zbus_serve_config* cfg, zbus_network* po
       most_form = std::max(most_form, form_extra(net));
       if (net->split_z.Z) slices += split_ops_bytes(net->n);
       if (net->split_zt.Z) slices += split_ops_bytes(net->n);
+      if (net->split_base) slices += split_scratch_bytes(net->n, net->split.rows);
     }
     if (slices > 0 && all + most_form + slices > ops_budget) {
       ZB_CUDA(cudaStreamSynchronize(st));
       for (auto net : nets) {
-        drop_graphs(net);
+        split_drop_scratch(net);
         split_release(&net->split_z);
         split_release(&net->split_zt);
       }

@@ -399,6 +399,7 @@ bool split_ready(zbus_network net, bool adjoint, cudaStream_t st);
 // Scratch for the split sweeps of up to B scenarios, at most what
 // SPLIT_SCRATCH_MAX holds: the scenarios per pass, 0 if memory does not do
 int64_t split_rows(zbus_network net, int64_t B);
+void split_drop_scratch(zbus_network net);   // no work of the network in flight
 bool use_graphs();   // false when ZBUS_NO_GRAPH=1 (sweeps launched from the host)
 // One sweep enqueued on a stream: the last kernel sets the WHILE condition
 // through h when use_handle; ev (or nullptr) brackets the kernels.
