@@ -99,6 +99,19 @@ __global__ void k_serve_done(const int32_t* __restrict__ iters, const uint8_t* _
     for (int j = threadIdx.x; j < n; j += blockDim.x) warm[j] = V[(int64_t)first * n + j];
 }
 
+// Forms the slices of Z again when the loop ends, for the networks that came
+// with them and hold their FP64 operands: the allocation-free solve, which
+// cannot form them, is to run as zbus_solve does (a device too full for them
+// leaves both on the FP64 contraction until it is not).
+struct SliceKeeper {
+  std::vector<zbus_network> nets;
+  cudaStream_t st;
+  ~SliceKeeper() {
+    for (auto net : nets)
+      if (net->Zr) split_ready(net, false, st);
+  }
+};
+
 struct Inflight {
   zbus_request req;
   int64_t s0;
@@ -191,9 +204,11 @@ extern "C" zbus_status zbus_serve(const zbus_serve_config* cfg, zbus_network* po
   const size_t ops_budget = budget - (size_t)per_slot * cap;
   // the slices the plain method keeps of each Z and the scratch of its sweeps
   // are no part of the cache: they stay only where they fit beside all of it
+  SliceKeeper keeper{{}, st};
   {
     size_t all = 0, most_form = 0, slices = 0;
     for (auto net : nets) {
+      if (net->split_z.Z) keeper.nets.push_back(net);
       all += cache_bytes(net, cfg->precision);
       most_form = std::max(most_form, form_extra(net));
       if (net->split_z.Z) slices += split_ops_bytes(net->n);

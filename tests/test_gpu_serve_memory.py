@@ -63,3 +63,31 @@ def test_sweep_scratch_outside_the_budget_is_given_back():
         V, it, cv = net.solve(sw, sd)
         assert cv.cpu().numpy().all()
         net.close()
+
+
+@pytest.mark.parametrize("evict", [False, True])
+def test_allocation_free_solve_after_a_tight_serving_loop(evict):
+    """The same bits as zbus_solve, whether the loop gave up only the slices
+    (no room beside the cache) or a network's operands in turn with the
+    other's, and formed them again."""
+    feeders, nets, loads, reqs, budget = pool_and_budget(1 << 20)
+    if evict:   # the cache holds the larger network's operands alone
+        budget -= zbus.zbus_serve_footprint(nets[0].handle, "fp16_scaled")[0] // 2
+    for _ in range(2):
+        zbus.serve(nets, reqs, max_slots=128, hbm_budget_bytes=budget)
+        for f, net, (sw, sd) in zip(feeders, nets, loads):
+            B = sw.shape[0]
+            out = torch.empty((B, f.n), dtype=torch.complex128, device="cuda")
+            it = torch.empty(B, dtype=torch.int32, device="cuda")
+            cv = torch.empty(B, dtype=torch.uint8, device="cuda")
+            try:
+                zbus.zbus_solve_noalloc(net.handle, sw, sd, None, 1e-8, 50, "maxabs", out, it, cv)
+            except zbus.ZbusError as e:    # evicted at the end: refused, not answered otherwise
+                assert evict and "zbus_network_reserve" in str(e)
+                continue
+            V, it2, cv2 = net.solve(sw, sd)
+            assert np.array_equal(out.cpu().numpy(), V.cpu().numpy())
+            assert np.array_equal(it.cpu().numpy(), it2.cpu().numpy())
+            assert np.array_equal(cv.cpu().numpy(), cv2.cpu().numpy())
+    for net in nets:
+        net.close()
