@@ -868,6 +868,19 @@ zbus_status split_parts(zbus_network net, const std::vector<int32_t>& ptr,
   return ZBUS_OK;
 }
 
+namespace {
+
+// One value for every size, so that calls of several host threads cannot lower
+// each other's.
+template <bool ADJ, bool FIRST>
+cudaError_t allow_step_smem() {
+  return cudaFuncSetAttribute(k_split_step<ADJ, FIRST>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              SPLIT_MAX_NPAD * (int)sizeof(double2));
+}
+
+}  // namespace
+
 zbus_status split_pack(SplitOps* ops, const double* Zr, const double* Zi, int n, int n_pad,
                        const int2* part, const int32_t* part_col, cudaStream_t st) {
   if (ops->Z) return ZBUS_OK;
@@ -876,6 +889,10 @@ zbus_status split_pack(SplitOps* ops, const double* Zr, const double* Zi, int n,
   ops->n_pad = n_pad;
   ops->part = part;
   ops->part_col = part_col;
+  ZB_CUDA((allow_step_smem<false, true>()));
+  ZB_CUDA((allow_step_smem<false, false>()));
+  ZB_CUDA((allow_step_smem<true, true>()));
+  ZB_CUDA((allow_step_smem<true, false>()));
   const int K = split_kpad(n);
   // N-tile: 192 or 256 outputs, whichever leaves less of the last tile idle
   ops->BN = round_up(n, 192) < round_up(n, 256) ? 192 : 256;
@@ -926,9 +943,6 @@ void launch_step(SolveCtx* ctx, const SplitOps& ops, const double2* w, int n, in
                  int64_t rows, cudaGraphConditionalHandle h, bool use_handle, cudaStream_t st) {
   const SplitRows m64 = {ops.Zr, ops.Zi, ops.part, ops.part_col, ops.n_pad};
   const size_t smem = (size_t)n * sizeof(double2);
-  if (smem > 32 * 1024)
-    cudaFuncSetAttribute(k_split_step<ADJ, FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
   k_split_step<ADJ, FIRST><<<step_grid(batch), step_threads(n), smem, st>>>(
       ctx, ops.zs, m64, w, n, split_kpad(n), rows, h, use_handle ? 1 : 0);
 }
