@@ -423,7 +423,9 @@ zbus_status zbus_power_mismatch(zbus_network net, int64_t B, const double* V,
  * kernel, the contraction and the convergence kernel; active[k] the number of
  * scenarios the sweep processed.  *sweeps receives the number of sweeps
  * launched (the loop runs max_iter sweeps; those after the last active one
- * have active[k] = 0).  Any output may be NULL.
+ * have active[k] = 0; a plain FP64 batch solved in passes of fewer scenarios
+ * has max_iter sweeps for each, one pass after the other).  Any output may be
+ * NULL.
  */
 zbus_status zbus_last_profile(zbus_network net, int32_t max_n, float* ms, int32_t* active,
                               int32_t* sweeps);

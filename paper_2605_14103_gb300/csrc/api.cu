@@ -686,7 +686,17 @@ zbus_status solve_split(zbus_network net, const SolveCtx& h, int64_t rows, bool 
                         cudaStream_t st) {
   const int n = net->n;
   net->last_ctx = net->ws.ctx;
+  Profile& P = net->prof;
+  const int64_t passes = (h.B + rows - 1) / rows;
+  if (profile) {   // the sweeps of one pass after those of the other
+    if (passes * h.max_iter > INT32_MAX / 4)
+      return fail(ZBUS_ERR_ARG, "too many sweeps to profile");
+    ZB_CHECK(ensure_profile(net, (int32_t)(passes * h.max_iter)));
+    ZB_CUDA(cudaMemsetAsync(P.d_hist, 0, (size_t)(passes * h.max_iter) * sizeof(int32_t), st));
+    P.sweeps = (int)(passes * h.max_iter);
+  }
   for (int64_t b0 = 0; b0 < h.B; b0 += rows) {
+    const int64_t k0 = b0 / rows * h.max_iter;   // the pass's first sweep
     const int64_t Bk = std::min<int64_t>(rows, h.B - b0);
     const int64_t o = b0 * n;
     SolveCtx hk = h;
@@ -700,9 +710,7 @@ zbus_status solve_split(zbus_network net, const SolveCtx& h, int64_t rows, bool 
     hk.B = (int32_t)Bk;
     hk.err = b0 > 0;
     if (profile) {
-      ZB_CHECK(ensure_profile(net, h.max_iter));
-      ZB_CUDA(cudaMemsetAsync(net->prof.d_hist, 0, (size_t)h.max_iter * sizeof(int32_t), st));
-      hk.hist = net->prof.d_hist;
+      hk.hist = P.d_hist + k0;
       hk.hist_n = h.max_iter;
     }
     launch_init(net->ws.ctx, hk, net->w, n, (int)Bk, st);
@@ -710,9 +718,7 @@ zbus_status solve_split(zbus_network net, const SolveCtx& h, int64_t rows, bool 
     ZB_CUDA(cudaGetLastError());
     if (profile) {
       for (int k = 0; k < h.max_iter; ++k)
-        ZB_CHECK(enqueue_sweep_split(net, Bk, 0, 0, false, st,
-                                     &net->prof.ev[(size_t)4 * k]));
-      net->prof.sweeps = h.max_iter;
+        ZB_CHECK(enqueue_sweep_split(net, Bk, 0, 0, false, st, &P.ev[(size_t)4 * (k0 + k)]));
     } else if (use_graphs()) {
       GraphEntry* g = nullptr;
       ZB_CHECK(get_while_graph(net, Bk, GRAPH_KEY_SPLIT, 0, enqueue_sweep_split, &g));
@@ -774,8 +780,7 @@ zbus_status solve_device(zbus_network net, int64_t B, const double* S_wye, const
   h.rule = o.conv_rule;
   h.ntn = net->n_pad / F64_BN;
   const int64_t rows = split_ready(net, false, st) ? split_rows(net, B) : 0;
-  if (rows > 0 && (rows >= B || o.profile != 1))
-    return solve_split(net, h, rows, o.profile == 1, st);
+  if (rows > 0) return solve_split(net, h, rows, o.profile == 1, st);
   const int grid = gemm_f64_grid((int)B, net->n_pad);
   if (o.profile == 1) {
     ZB_CHECK(ensure_profile(net, max_iter));

@@ -59,6 +59,15 @@ def main():
             for p, q in zip(x, y):
                 assert np.array_equal(p.cpu().numpy(), q.cpu().numpy()), (B, rows, rule)
             assert few.device_status() == 0
+            # the profile is of these passes
+            few.solve(Sw, Sd, rule=rule, max_iter=20, profile=True)
+            torch.cuda.synchronize()
+            ms, active = few.last_profile()
+            counts = want[1].astype(int)
+            assert len(ms) == len(active) == 20 * -(-B // rows) and (ms >= 0).all()
+            for p in range(-(-B // rows)):
+                mine = counts[p * rows:(p + 1) * rows]
+                assert list(active[20 * p:20 * p + 20]) == [(mine > k).sum() for k in range(20)]
             few.close()
             one.close()
     _, word = zbus.zbus_checked_status()
