@@ -209,7 +209,7 @@ k_gemm3m_f64(const SolveCtx* __restrict__ ctx, const double* __restrict__ Zr,
             const double2 wi = w ? w[i] : vo;
             const double2 vn = make_double2(wi.x + dr, wi.y + di);
             V[g] = vn;
-            double step = hypot(vn.x - vo.x, vn.y - vo.y);
+            double step = step_length(vn.x - vo.x, vn.y - vo.y);
             if (step != step) step = INFINITY;
             dmax = fmax(dmax, step);
             if (summag) dsum += hypot(vn.x, vn.y) - hypot(vo.x, vo.y);
@@ -287,7 +287,7 @@ k_gemm3m_f64_small(const SolveCtx* __restrict__ ctx, const double* __restrict__ 
       const double2 wi = w ? w[i] : vo;
       const double2 vn = make_double2(wi.x + dr, wi.y + di);
       V[g] = vn;
-      double step = hypot(vn.x - vo.x, vn.y - vo.y);
+      double step = step_length(vn.x - vo.x, vn.y - vo.y);
       if (step != step) step = INFINITY;
       dm = step;
       ds = hypot(vn.x, vn.y) - hypot(vo.x, vo.y);
@@ -324,10 +324,9 @@ k_gemm3m_f64_small(const SolveCtx* __restrict__ ctx, const double* __restrict__ 
 // value is formed with the arithmetic of the sweep kernels: the load currents
 // of bus_injection (a thread per unknown draws its wye current or its bus's
 // delta branch, then adds the branches into its phase as bus_injection does),
-// each output's three products summed over k in sequence, so the voltages are
-// bitwise those of the sweep-per-launch path.  (The stop test compares the
-// root of the largest squared step with tol, theirs the largest hypot: equal
-// to an ulp.)
+// each output's three products summed over k in sequence, the step lengths of
+// step_length (the root of the largest square is the largest root), so the
+// results are bitwise those of the sweep-per-launch path.
 //
 // Bound by the FP64 pipe, which a warp's instruction holds as long for 12
 // lanes as for 32: each of the three products of an output has a thread of

@@ -13,6 +13,16 @@ __device__ __forceinline__ bool has_load(double2 S) {
   return ((__double_as_longlong(S.x) | __double_as_longlong(S.y)) << 1) != 0;
 }
 
+// Length of a voltage step, as every stop test of the plain method forms it:
+// the root of the rounded square, hypot where the square leaves the range.
+// Never decreasing in the square, so a kernel may compare squares and take one
+// root.
+__device__ __forceinline__ double step_length(double dx, double dy) {
+  const double q = fma(dx, dx, dy * dy);
+  const unsigned ex = (unsigned)(__double_as_longlong(q) >> 52);   // q >= 0 or NaN
+  return (ex & 0x7FF) - 128u < 1792u ? sqrt(q) : hypot(dx, dy);
+}
+
 // conj(S / v) = conj(S) v / |v|^2; zero when the slot has no load.  The
 // multiply-adds are written out, so every kernel rounds alike.
 __device__ __forceinline__ double2 load_draw(double2 S, double2 v) {
