@@ -18,7 +18,8 @@
 // leading digits of |Re| + |Im| (8 bits, rounded down), the sum of magnitudes
 // in units of the two scales.  Rows where it is below SPLIT_WEAK are formed in
 // FP64 by the step kernel, from the matrix and the operand themselves, over
-// the unknowns of the row's own part of the network.
+// the unknowns of the row's own part of the network; a row of the plain sweep
+// only if the digits' error could show beside the rounding of its voltage.
 //
 // Why: this GPU does 1.25 TFLOP/s in FP64 and about 1.9 PFLOP/s in FP16; the
 // 28 digit products of 6 n^2 operations each are 168 n^2 operations at 1500
@@ -298,7 +299,7 @@ k_split_gemm(SolveCtx* __restrict__ ctx, const __grid_constant__ CUtensorMap tmX
             if (lane == 0) mbar_arrive(&tempty[buf]);
           }
 #pragma unroll
-          for (int t = 0; t < 32; ++t) acc[c * 32 + t] += __float2int_rn(v[t]);
+          for (int t = 0; t < 32; ++t) acc[c * 32 + t] += __float2int_ru(v[t]);
         }
       }
       const int64_t row = (int64_t)it.mt * BM + q * 32 + lane;
@@ -353,7 +354,8 @@ __device__ __forceinline__ long long fixed_point(double x, int e) {
 // Slices of one row of n complex values, by all threads of the block: digit p
 // of component c of value(j) goes to plane c * 7 + p of out, `plane` halves
 // apart, the leading digits of |Re| + |Im| to plane 21; a thread takes four
-// columns of one component at a time.
+// columns of one component at a time.  A magnitude below one digit is 2^-12, so
+// that a sum of products is zero (rounded up, k_split_gemm) only where each is.
 template <typename Load>
 __device__ __forceinline__ void write_slices(Load value, int n, int K_pad, int e, __half* out,
                                              int64_t plane) {
@@ -363,6 +365,7 @@ __device__ __forceinline__ void write_slices(Load value, int n, int K_pad, int e
     const int c = u / groups, g = u - c * groups;
     long long y[4];
     uint32_t mag[2] = {0x65006500u, 0x65006500u};   // 1280 + the magnitude's digit
+    uint32_t tiny[2] = {0u, 0u};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int j = g * 4 + i;
@@ -370,7 +373,9 @@ __device__ __forceinline__ void write_slices(Load value, int n, int K_pad, int e
       y[i] = fixed_point(c == 1 ? v.y : v.x, e);
       if (c == 2) {
         const long long im = fixed_point(v.y, e);
-        mag[i >> 1] += (uint32_t)((llabs(y[i]) + llabs(im)) >> (SPLIT_BITS - 7)) << (16 * (i & 1));
+        const uint32_t d = (uint32_t)((llabs(y[i]) + llabs(im)) >> (SPLIT_BITS - 7));
+        mag[i >> 1] += d << (16 * (i & 1));
+        if (d == 0 && has_load(v)) tiny[i >> 1] |= 0x0C00u << (16 * (i & 1));   // 2^-12
         y[i] += im;
       }
     }
@@ -379,7 +384,7 @@ __device__ __forceinline__ void write_slices(Load value, int n, int K_pad, int e
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const __half2 hv = __hsub2(*reinterpret_cast<const __half2*>(&mag[i]), bias);
-        mag[i] = *reinterpret_cast<const uint32_t*>(&hv);
+        mag[i] = *reinterpret_cast<const uint32_t*>(&hv) | tiny[i];   // of a half that is 0
       }
       *reinterpret_cast<uint2*>(dst + SPLIT_S * plane) = make_uint2(mag[0], mag[1]);
     }
@@ -507,23 +512,22 @@ struct SplitRows {
   const int2* part;
   const int32_t* part_col;
   int n_pad;
+  __device__ int size(int j) const {   // unknowns of j's part
+    const int2 r = __ldg(part + j);
+    return r.y - r.x;
+  }
 };
 
-// The weak rows of a warp (lane's: j0 + lane; `weak`, one bit each) in FP64,
-// four at a time, eight lanes a row over the unknowns of its part: in (re, im)
-// of their lanes.  x: the operand.  Columns without current cost no arithmetic.
-__device__ __noinline__ double2 weak_rows(unsigned weak, int j0, int n, const SplitRows& m,
-                                          const double2* x) {
+// The block's weak rows (list, cnt of them) in FP64, over the unknowns of their
+// parts, into out[row]; x: the operand.  Four rows a warp, eight lanes a row:
+// most are of parts of a few buses.  Columns without current cost no
+// arithmetic.
+__device__ __noinline__ void weak_rows(const uint16_t* list, int cnt, int n, const SplitRows& m,
+                                       const double2* x, double2* out) {
   const int lane = threadIdx.x & 31;
-  double2 mine = make_double2(0.0, 0.0);
-  while (weak) {
-    int bit[4], row = -1;
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      bit[g] = __ffs(weak) - 1;   // -1: none left
-      weak &= weak - 1;
-      if (lane >> 3 == g && bit[g] >= 0) row = j0 + bit[g];
-    }
+  for (int r0 = (threadIdx.x >> 5) * 4; r0 < cnt; r0 += blockDim.x >> 3) {
+    const int r = r0 + (lane >> 3);
+    const int row = r < cnt ? list[r] : -1;
     double2 a = make_double2(0.0, 0.0);
     if (row >= 0) {
       const int2 cols = __ldg(m.part + row);
@@ -542,14 +546,17 @@ __device__ __noinline__ double2 weak_rows(unsigned weak, int j0, int n, const Sp
       a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
       a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
     }
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      const double re = __shfl_sync(0xffffffffu, a.x, 8 * g);
-      const double im = __shfl_sync(0xffffffffu, a.y, 8 * g);
-      if (lane == bit[g]) mine = make_double2(re, im);
-    }
+    if (row >= 0 && (lane & 7) == 0) out[row] = a;
   }
-  return mine;
+}
+
+// Whether the digits' error in a row of scale s with m terms, some 2^-55.6 sqrt(m)
+// of 2^62 s, is within 2^-57 of the larger part of its new voltage, whose own rounding is
+// some 2^-54.8 of it: by the exponents.
+__device__ __forceinline__ bool beside_voltage(double s, double vx, double vy, int m) {
+  const int es = __double2hiint(s) >> 20;
+  const int ev = max(__double2hiint(vx) & 0x7FFFFFFF, __double2hiint(vy) & 0x7FFFFFFF) >> 20;
+  return es <= ev - 64 - (33 - __clz(m)) / 2;
 }
 
 // Blocks of 256 threads an SM holds: at 2 the FP64 pipe waits (176 us a sweep
@@ -563,11 +570,14 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs, SplitRow
              const double2* __restrict__ w, int n, int K_pad, int64_t rows,
              cudaGraphConditionalHandle h, int use_handle) {
   extern __shared__ double2 op[];   // [n] operand of the next sweep
+  uint16_t* const weak = reinterpret_cast<uint16_t*>(op + n);   // [n] rows for FP64
   __shared__ unsigned long long red[8];
   __shared__ double sred[8];
-  __shared__ int s_keep, s_slot;
+  __shared__ int s_keep, s_slot, s_weak;
   const SolveCtx& c = *ctx;
   const int tid = threadIdx.x;
+  if (tid == 0) s_weak = 0;
+  __syncthreads();
   const int ld = (n + 7) & ~7;
   const int nb = (n + 2) / 3;
   const int par = c.iter & 1;
@@ -590,13 +600,27 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs, SplitRow
     double dsum = 0.0;
     const double xb = FIRST ? 0.0 : xs[slot];
     const double inv_s = ADJ ? 1.0 / c.gscale[in ? b : 0] : 0.0;
-    // voltages, a thread per unknown (whole warps)
+    // the new voltage, step and magnitudes of unknown j: w_j + s (re, im)
+    const auto update = [&](int j, double re, double im, double s, double2 vo, double2 wj) {
+      const double2 v = make_double2(fma(re, s, wj.x), fma(im, s, wj.y));
+      V[j] = v;
+      op[j] = v;
+      const double dx = v.x - vo.x, dy = v.y - vo.y;
+      const unsigned long long qb = abs_bits(fma(dx, dx, dy * dy));
+      if ((unsigned)(qb >> 52) - 128u < 1792u) {   // far inside the range of squares
+        st2 = max_u64(st2, qb);
+      } else if ((abs_bits(dx) | abs_bits(dy)) != 0ull) {
+        const unsigned long long hb = abs_bits(hypot(dx, dy));
+        sth = max_u64(sth, hb > 0x7FF0000000000000ull ? 0x7FF0000000000000ull : hb);
+      }
+      if (summag) dsum += hypot(v.x, v.y) - hypot(vo.x, vo.y);
+    };
+    unsigned long long mine = 0ull;      // this thread's weak rows, a bit an iteration
+    // voltages, a thread per unknown
     if (in)
-      for (int j0 = tid & ~31; j0 < n; j0 += blockDim.x) {
-        const bool own = j0 + (tid & 31) < n;
-        const int j = own ? j0 + (tid & 31) : n - 1;
+      for (int j = tid, i = 0; j < n; j += blockDim.x, ++i) {
         if (FIRST) {
-          if (own) op[j] = V[j];
+          op[j] = V[j];
           continue;
         }
         const int32_t* D = c.D + (int64_t)slot * ld + j;
@@ -606,10 +630,10 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs, SplitRow
         for (int q = 0; q < 3; ++q)
 #pragma unroll
           for (int d = 0; d < SPLIT_S; ++d) t[q][d] = D[(q * SPLIT_S + d) * plane];
-        const bool low = D[3 * SPLIT_S * plane] < SPLIT_WEAK;
+        const int mag = D[3 * SPLIT_S * plane];
         const double2 vo = V[j];
         const double2 wj = ADJ ? make_double2(0.0, 0.0) : w[j];
-        double s = zs[j] * xb;
+        const double s = zs[j] * xb;
         long long hi[3], lo[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
@@ -617,34 +641,30 @@ k_split_step(SolveCtx* __restrict__ ctx, const double* __restrict__ zs, SplitRow
                   ((long long)t[q][2] << 8) + t[q][3];
           lo[q] = ((long long)t[q][4] << 16) + ((long long)t[q][5] << 8) + t[q][6];
         }
-        double re = recombine(hi[0] - hi[1], lo[0] - lo[1]);
-        double im = recombine(hi[2] - hi[0] - hi[1], lo[2] - lo[0] - lo[1]);
-        // a scale of zero (no current at all) or one that is not a number
-        // gives every row its value
-        const unsigned weak = __ballot_sync(0xffffffffu, own && low && xb > 0.0);
-        if (weak) {
-          const double2 f = weak_rows(weak, j0, n, m64, xop);
-          if (weak >> (tid & 31) & 1) {
-            re = f.x;
-            im = f.y;
-            s = 1.0;
-          }
+        const double re = recombine(hi[0] - hi[1], lo[0] - lo[1]);
+        const double im = recombine(hi[2] - hi[0] - hi[1], lo[2] - lo[0] - lo[1]);
+        // a sum of zero is exact; a scale that is not a number goes to every row
+        if (mag > 0 && mag < SPLIT_WEAK && xb > 0.0 &&
+            (ADJ || !beside_voltage(s, fma(re, s, wj.x), fma(im, s, wj.y), m64.size(j)))) {
+          mine |= 1ull << i;
+          weak[atomicAdd(&s_weak, 1)] = (uint16_t)j;
+        } else {
+          update(j, re, im, s, vo, wj);
         }
-        if (!own) continue;
-        const double2 v = make_double2(fma(re, s, wj.x), fma(im, s, wj.y));
-        V[j] = v;
-        op[j] = v;
-        const double dx = v.x - vo.x, dy = v.y - vo.y;
-        const unsigned long long qb = abs_bits(fma(dx, dx, dy * dy));
-        if ((unsigned)(qb >> 52) - 128u < 1792u) {   // far inside the range of squares
-          st2 = max_u64(st2, qb);
-        } else if ((abs_bits(dx) | abs_bits(dy)) != 0ull) {
-          const unsigned long long hb = abs_bits(hypot(dx, dy));
-          sth = max_u64(sth, hb > 0x7FF0000000000000ull ? 0x7FF0000000000000ull : hb);
-        }
-        if (summag) dsum += hypot(v.x, v.y) - hypot(vo.x, vo.y);
       }
     if (!FIRST) {
+      __syncthreads();
+      const int cnt = s_weak;
+      if (cnt > 0) {
+        weak_rows(weak, cnt, n, m64, xop, op);
+        __syncthreads();
+        for (int j = tid; mine; j += blockDim.x, mine >>= 1)
+          if (mine & 1ull) {
+            const double2 d = op[j];
+            update(j, d.x, d.y, 1.0, V[j], ADJ ? make_double2(0.0, 0.0) : w[j]);
+          }
+        if (tid == 0) s_weak = 0;
+      }
       st2 = block_max_u64(st2, red);
       sth = block_max_u64(sth, red);
       if (summag) {
@@ -802,6 +822,9 @@ zbus_status launch_gemm(SolveCtx* ctx, const SplitScratch& s, const SplitOps& op
   return ZBUS_OK;
 }
 
+// Operand and list of a block: 16 and 2 bytes an unknown.
+size_t step_smem(int n) { return (size_t)n * (sizeof(double2) + sizeof(uint16_t)); }
+
 int step_threads(int n) { return n <= 3 * 160 ? 128 : 256; }
 
 int step_grid(int64_t batch) {
@@ -876,7 +899,7 @@ template <bool ADJ, bool FIRST>
 cudaError_t allow_step_smem() {
   return cudaFuncSetAttribute(k_split_step<ADJ, FIRST>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              SPLIT_MAX_NPAD * (int)sizeof(double2));
+                              (int)step_smem(SPLIT_MAX_NPAD));
 }
 
 }  // namespace
@@ -942,8 +965,7 @@ template <bool ADJ, bool FIRST>
 void launch_step(SolveCtx* ctx, const SplitOps& ops, const double2* w, int n, int64_t batch,
                  int64_t rows, cudaGraphConditionalHandle h, bool use_handle, cudaStream_t st) {
   const SplitRows m64 = {ops.Zr, ops.Zi, ops.part, ops.part_col, ops.n_pad};
-  const size_t smem = (size_t)n * sizeof(double2);
-  k_split_step<ADJ, FIRST><<<step_grid(batch), step_threads(n), smem, st>>>(
+  k_split_step<ADJ, FIRST><<<step_grid(batch), step_threads(n), step_smem(n), st>>>(
       ctx, ops.zs, m64, w, n, split_kpad(n), rows, h, use_handle ? 1 : 0);
 }
 
