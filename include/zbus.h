@@ -59,7 +59,10 @@ typedef enum {
 } zbus_status;
 
 typedef enum {
-  ZBUS_FP64 = 0,              /* plain map, FP64 on the CUDA cores */
+  ZBUS_FP64 = 0,              /* plain map in FP64; from 97 to 12288 unknowns the
+                                 products with Z run as sums of products of
+                                 8-bit digits on the tensor cores, a row's
+                                 error within that of an FP64 sum of its terms */
   ZBUS_MIXED_BF16X2 = 1,      /* defect form, Z as BF16 hi+lo on tensor cores */
   ZBUS_MIXED_FP16_SCALED = 2, /* defect form, Z as row-scaled FP16 hi+lo */
   ZBUS_TREE_SWEEP = 3         /* defect form, Z applied as a backward / forward
@@ -128,6 +131,10 @@ void zbus_solve_opts_default(zbus_solve_opts* opts);
  *   v_slack_reim  host double[6], complex slack phase voltages (pu)
  *   cuda_stream   stream for the setup work; the call returns after it finished
  *   out           receives the handle (owned by the library until destroy)
+ *
+ * The handle holds about 16 n^2 (Z) + 24 n^2 (its FP64 operands) bytes and, for
+ * the plain form from 97 unknowns, 44 n^2 of digits of Z (left out where the
+ * device does not hold them: the FP64 contraction runs until it does).
  *
  * Returns ZBUS_ERR_SINGULAR if a pivot is zero or not finite, ZBUS_ERR_OOM if
  * device memory runs out.
@@ -203,7 +210,12 @@ zbus_status zbus_network_reserve(zbus_network net, int64_t B, int32_t precision)
  *                   modes, the FP64 mismatch test passed)
  *   cuda_stream     all work is enqueued on this stream; results are valid
  *                   after it synchronises.  Scratch grows on demand (a
- *                   synchronous allocation) unless reserved beforehand.
+ *                   synchronous allocation) unless reserved beforehand.  The
+ *                   plain form from 97 unknowns takes about 148 n bytes a
+ *                   scenario beside it, up to 8 GiB or what the device holds
+ *                   (a larger batch runs in passes, with the same bits), kept
+ *                   until the handle goes or a serving loop's budget has no
+ *                   room for them.
  *
  * The array arguments are all device memory or all host memory (pinned or
  * pageable; a mix returns ZBUS_ERR_ARG).  With host memory the batch is
@@ -446,7 +458,12 @@ zbus_status zbus_last_profile(zbus_network net, int32_t max_n, float* ms, int32_
  * process exits, and this call itself loads nothing.  The network must exist
  * already (create it at start-up, before any stream capture).  The sweeps are
  * launched from the host (max_iter sweeps; once no scenario is active the
- * remaining launches return at once).
+ * remaining launches return at once).  From 97 unknowns the digits of the
+ * tensor-core products take more of the array than the limit below is for
+ * (about 148 n bytes per scenario): such a batch runs in passes of the
+ * scenarios that fit, max_iter sweeps each, with the same bits.  Where the
+ * device did not hold the digits of Z (zbus_network_create), this call takes
+ * the FP64 contraction and agrees with zbus_solve to rounding only.
  *
  *   arguments as zbus_solve, with conv_rule (zbus_conv_rule) in place of
  *   opts, but device memory only: a host array (pinned or pageable) returns
@@ -454,8 +471,8 @@ zbus_status zbus_last_profile(zbus_network net, int32_t max_n, float* ms, int32_
  *   when the batch needs more than the 16 MiB: about 16 MiB / (24 n_pad +
  *   16 ceil(n/48) + 5) bytes per scenario, n_pad = n rounded up to a multiple
  *   of 48 (about 1790 scenarios for n = 381).  Partial-phase networks:
- *   ZBUS_ERR_UNSUPPORTED.  After this call zbus_last_device_status reports
- *   ZBUS_OK (the FP64 sweeps have no device-side waits).
+ *   ZBUS_ERR_UNSUPPORTED.  zbus_last_device_status reports this call's waits
+ *   as those of zbus_solve.
  *
  * All calls share the array and it keeps the last call's contents; every call
  * rewrites what it reads, but calls that overlap on the GPU (other streams or
@@ -481,7 +498,7 @@ zbus_status zbus_solve_noalloc(zbus_network net, int64_t B,
  * slot j: A_jj = conj(S_j / v_j^2), D_jj = -1 / conj(v_j); delta branch
  * x -> y, u = v_x - v_y: conj(S / u^2) in A on (x,x), (y,y) and its negative on
  * (x,y), (y,x); -1 / conj(u), +1 / conj(u) at rows x, y of D).  FP64 throughout
- * (the 3M contraction of the plain method with Z^T); the sweeps run in a
+ * (the contraction of the plain method with Z^T); the sweeps run in a
  * device-side loop like the solve.
  *
  * Complex gradients follow the convention of complex autograd:
@@ -516,10 +533,10 @@ zbus_status zbus_solve_noalloc(zbus_network net, int64_t B,
  *   cuda_stream     all work is enqueued on this stream
  *
  * Device buffers only (ZBUS_ERR_ARG otherwise).  The first call on a network
- * forms Z^T (three n_pad x n_pad FP64 arrays kept with the handle); scratch
- * grows on demand (synchronous).  Shares the handle's solve scratch, so it
- * must not overlap a solve of the same handle on another stream.  Works on
- * partial-phase networks.  B = 0 is a no-op.
+ * forms Z^T (three n_pad x n_pad FP64 arrays and its digits kept with the
+ * handle); scratch grows on demand (synchronous).  Shares the handle's solve
+ * scratch, so it must not overlap a solve of the same handle on another stream.
+ * Works on partial-phase networks.  B = 0 is a no-op.
  */
 zbus_status zbus_solve_adjoint(zbus_network net, int64_t B,
                                const double* S_wye, const double* S_delta,
@@ -534,11 +551,13 @@ zbus_status zbus_solve_adjoint(zbus_network net, int64_t B,
  * zbus_last_device_status -- the errors the device detected during the last
  * solve on net (the error word its kernels set instead of hanging or
  * faulting).  Synchronises cuda_stream first, so the solve must have been
- * enqueued on it.  ZBUS_OK if the solve ran clean (or was FP64, which has no
- * device-side waits); ZBUS_ERR_TIMEOUT if a bounded wait of the tensor-core
- * pipeline gave up (its results are then not to be used); ZBUS_ERR_DEVICE
- * for any other error word.  The next solve clears the word.  Project-
- * written; the paper has no counterpart.
+ * enqueued on it.  ZBUS_OK if the solve ran clean; ZBUS_ERR_TIMEOUT if a
+ * bounded wait of a tensor-core pipeline gave up, in any form including the
+ * plain FP64 one and the dense gradient (the scenarios still active then are
+ * not flagged as converged, and their results not to be used); ZBUS_ERR_DEVICE
+ * for any other error word.  Each network keeps its own word; its next solve or
+ * gradient clears it (of a solve of host arrays, each chunk of the batch
+ * does).  Project-written; the paper has no counterpart.
  */
 zbus_status zbus_last_device_status(zbus_network net, void* cuda_stream);
 
@@ -647,7 +666,7 @@ zbus_status zbus_nr_solve(zbus_nr_network net, int64_t B, const double* P, const
  * nodes, maps, permutations, level lists) is tested against its buffer
  * before use; a bad one records a code (0x1nn plain FP64 kernels, 0x2nn
  * tensor-core and tree engine, 0x3nn load gradient, 0x4nn Newton-Raphson,
- * 0x5nn partial-phase maps) and the access is skipped instead of faulting.
+ * 0x5nn partial-phase maps, 0x6nn digit sweeps of the plain form) and the access is skipped instead of faulting.
  * *word (may be NULL) receives the first code recorded since the last call,
  * 0 if none (always 0 in the normal build), and the codes are cleared.
  * Synchronises the current device.  Project-written: the paper has no

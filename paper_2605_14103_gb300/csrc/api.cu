@@ -751,7 +751,7 @@ zbus_status solve_device(zbus_network net, int64_t B, const double* S_wye, const
   }
 
   net->last_group = nullptr;
-  net->last_ctx = nullptr;   // the sweeps on the CUDA cores have no device-side waits
+  net->last_ctx = nullptr;   // set by the path with device-side waits (solve_split)
   if (o.profile != 1 && net->n_pad <= FUSED_MAX_NPAD) {
     // a small feeder: the whole solve in one launch, a block per scenario
     // (bitwise the results of the sweep-per-launch path below)
