@@ -559,6 +559,10 @@ __host__ __device__ constexpr int shared_doubles(int m) {
 // pass's update and the second pass's products.  Every sum keeps its order.
 // 1000 scenarios: 2224 buses FP64 22.4 -> 15.3 ms, mixed 11.3 -> 6.6 ms; 118
 // buses mixed 1.14 -> 0.73 ms; one scenario of 2224 buses, FP64, 12.3 -> 6.3.
+// Larger grids, to which NR_TAIL_ROWS and NR_MIN_CTAS were not fitted, 1 and 500
+// scenarios of 5000 buses: FP64 33.2 -> 17.6 and 49.2 -> 33.6 ms, mixed 22.6 ->
+// 10.3 and 31.9 -> 16.2; 1 and 200 of 13659 (20 steps, 1500 products): FP64 3.64
+// -> 2.47 and 11.1 -> 7.86 s, mixed 2.34 -> 1.47 and 4.28 -> 3.19.
 template <class T>
 __global__ void __launch_bounds__(NR_THREADS, NR_MIN_CTAS) k_nr_solve(NrDev d, SolveArgs a) {
   constexpr bool MIXED = sizeof(T) == 4;

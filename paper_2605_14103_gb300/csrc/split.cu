@@ -26,8 +26,8 @@
 // times the rate.
 //
 // Measured per sweep against the FP64 contraction (k_currents_f64 +
-// k_gemm3m_f64 + the stop test): 1000 scenarios of 3069 unknowns 66 -> 1.32 ms
-// (contraction 1.03), 4096 of 381 3.5 -> 0.23 ms (0.085).
+// k_gemm3m_f64 + the stop test): 1000 scenarios of 3069 unknowns 66 -> 1.29 ms
+// (contraction 1.03), 4096 of 381 3.5 -> 0.23 ms (0.091).
 //
 // One sweep is two kernels: k_split_gemm (the 22 partial products of every
 // active scenario) and k_split_step (recombination, update, stop test, active
@@ -50,13 +50,15 @@ using namespace tc;
 
 constexpr int GEMM_THREADS = 320;      // TMA, MMA and eight epilogue warps
 // Least sum of leading digits (unit 2^-14 of the product of the scales) of a
-// row that keeps its digit products: 1.5.  Root mean square error of a row
-// over that of the FP64 contraction, by this sum (99 and 255 unknowns; loads
-// and upstream gradients of one size, one bus of 100 or 10^4 times the others,
-// sizes over twelve decades): below 0.25 4 to 10^4, 0.5 to 0.75 1.0 to 2.4, 1 to
-// 1.25 1.0 to 1.5, 1.25 to 1.5 1.0 to 1.25, 1.5 to 2 0.8 to 1.15, above 2 at
-// most 0.95.  With loads of one size the rows below are those of the small
-// parts, a few buses behind a line of their own at the slack.
+// row that keeps its digit products: 1.5.  Root mean square error of a row over
+// that of the FP64 contraction, by this sum (99 and 255 unknowns; loads and
+// upstream gradients of one size, one bus of 100 or 10^4 times the others, sizes
+// over twelve decades): below 0.25 4 to 10^4, 0.5 to 0.75 1.0 to 2.4, 1 to 1.25
+// 1.0 to 1.5, 1.25 to 1.5 1.0 to 1.25, 1.5 to 2 0.8 to 1.15, above 2 at most 0.95
+// (0.1 at 32, where most rows of a large feeder are).  With loads of one size the
+// rows below are those of the small parts, a few buses behind a line of their own
+// at the slack; the gradient of 4096 scenarios of 128 buses takes 5.52 ms without
+// them, 5.67 so and 5.93 with the line at 2.
 constexpr int SPLIT_WEAK = 3 << 13;
 constexpr int EPI_WARPS = 8;
 constexpr int TMEM_COLS = 512;         // two accumulators of up to 256 columns
@@ -126,8 +128,8 @@ __device__ __forceinline__ int split_deal(int round) {
 // half of the columns).  The accumulator is drained before its sum can pass
 // 2^24 (split_chunk) into 32-bit integer registers, the next chunk's MMAs running meanwhile in
 // the other accumulator.  Bound by the tensor pipe at large batches: 16384
-// scenarios of 3069 unknowns in 13.9 ms, 1.86 PFLOP/s of digit products (0.98
-// of the measured cuBLAS rate); a few scenarios read the 400 MB of slices of
+// scenarios of 3069 unknowns in 14.1 ms, 1.87 PFLOP/s of digit products (0.98
+// of the measured cuBLAS rate); a few scenarios read the 415 MB of slices of
 // Z once per sweep (0.15 ms).  Every wait is bounded as in k_contract_group, and
 // a block that gives up records its code and leaves nothing in flight.
 // ---------------------------------------------------------------------------
@@ -463,8 +465,8 @@ k_split_pack(const double* __restrict__ Zr, const double* __restrict__ Zi, int n
 // between runs; no result depends on it.
 //
 // Bound by the FP64 pipe (about 34 operations an unknown at two a clock and
-// SM: 91 us for 4096 scenarios of 381 unknowns; 74 % busy) and by the
-// latencies between the block's barriers: 143 us there, 203 before the
+// SM: 91 us for 4096 scenarios of 381 unknowns; 75 % busy) and by the
+// latencies between the block's barriers: 136 us there, 203 before the
 // voltages had a thread per unknown and the slices one per four columns, 156
 // before the tests for absent loads left the FP64 pipe.
 // ---------------------------------------------------------------------------
@@ -560,7 +562,8 @@ __device__ __forceinline__ bool beside_voltage(double s, double vx, double vy, i
 }
 
 // Blocks of 256 threads an SM holds: at 2 the FP64 pipe waits (176 us a sweep
-// of 4096 scenarios of 381 unknowns against 156, with comparisons on it), at 4 the spills cost a few
+// of 4096 scenarios of 381 unknowns against 156, with comparisons on it), at 4
+// the spills cost a few
 // scenarios (92 us a sweep of 16 of 3069 unknowns against 76).
 constexpr int STEP_MIN = 3;
 
