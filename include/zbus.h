@@ -399,7 +399,11 @@ typedef struct {
  * feeder's operands can be formed on the device (Z_LL^-1 again by
  * Gauss-Jordan, then its copies), and waits while they cannot; requests of
  * other feeders are admitted meanwhile.  Released operands of a pool network
- * are formed again on demand by any later call that needs them.  Each feeder
+ * are formed again on demand by any later call that needs them.  What the plain
+ * form keeps of the pool's networks (the digits of Z and the scratch of its
+ * sweeps) stays only where it fits beside all of that; otherwise it is
+ * released, and the digits are formed again when the loop ends for the
+ * networks that then hold their FP64 operands.  Each feeder
  * keeps its last converged voltage for warm starts.  Runs on the calling
  * thread; the callbacks run on it too.
  */
