@@ -91,9 +91,9 @@ __device__ __forceinline__ void st_i8(int32_t* p, const int* v) {
 // ---------------------------------------------------------------------------
 // Work of the contraction: one item is the 128 x BN block (mt, nt) of one
 // partial product (c, d): component c (Re, Im, Re + Im; 3, the magnitudes, has
-// one digit) and digit weight d, the sum over p <= d of X_p Z_{d-p}^T.  Items are listed from the longest
-// (d = 6) to the shortest and dealt to the blocks back and forth, so every
-// block gets about the same number of k-blocks.
+// one digit) and digit weight d, the sum over p <= d of X_p Z_{d-p}^T.  Items
+// are listed from the longest (d = 6) to the shortest and dealt to the blocks
+// back and forth, so every block gets about the same number of k-blocks.
 // ---------------------------------------------------------------------------
 struct SplitItem {
   int c, d, mt, nt;
